@@ -1,0 +1,60 @@
+// Operand layout and digit arithmetic of the FP64 tensor-core GEMM
+// (k_gemm_f64tc.cu), shared with the sampler that writes its trajectory
+// operand.
+#pragma once
+
+#include <cstdint>
+
+namespace gbs {
+namespace f64tc {
+
+constexpr int kDigits = 7;        // balanced base-256 digits of a 56-bit fixed-point number
+constexpr int kTrajTile = 32;     // trajectories per tile, two sub-tiles of 16
+// one K step of 16 input modes: digit q of a 128-row A tile, of a 32-row
+// (16 alpha, 16 beta) B sub-tile
+constexpr int kASlice = 128 * 32;
+constexpr int kAStage = kDigits * kASlice;
+constexpr int kBSlice = 32 * 32;
+constexpr int kBSub = kDigits * kBSlice;
+constexpr int kBStage = 2 * kBSub;
+// scales beyond 2^+-kExpRange are left to the SIMT kernel
+constexpr int kExpRange = 400;
+constexpr int kExpNone = -(1 << 20);
+
+// Byte offset of (row, k) within a slice of one 16-wide K step: 8-row groups
+// of 256 bytes, each two core matrices of 8 rows x 16 bytes.
+__host__ __device__ __forceinline__ int core_offset(int row, int k) {
+    return (row >> 3) * 256 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
+}
+
+// v 2^s rounded to an integer (to nearest, halves away from zero), for
+// |v 2^s| <= 2^55 and a normal v; 0 below one half.
+__device__ __forceinline__ int64_t to_fixed(double v, int s) {
+    const int64_t bits = __double_as_longlong(v);
+    const int ex = (int)((bits >> 52) & 0x7ff) - 1075 + s;  // |v| 2^s = m 2^ex
+    const int64_t m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
+    int64_t x;
+    if (ex >= 0) x = m << ex;
+    else if (ex < -54) x = 0;
+    else x = ((m >> (-ex - 1)) + 1) >> 1;
+    return bits < 0 ? -x : x;
+}
+
+// The seven balanced digits of x (|x| <= 2^55) as BF16 bits, most significant
+// first: bytes of x + 128 (1 + 256 + ...), less 128.
+__device__ __forceinline__ void digits_bf16(int64_t x, uint16_t (&d)[kDigits]) {
+    const int64_t y = x + 0x808080808080ll;
+    d[0] = (uint16_t)(__float_as_uint((float)(int)(y >> 48)) >> 16);
+#pragma unroll
+    for (int q = 1; q < kDigits; ++q) {
+        const uint32_t b = (uint32_t)(y >> (8 * (kDigits - 1 - q))) & 255u;
+        // 2^23 + b, less 2^23 + 128: exact
+        d[q] = (uint16_t)(__float_as_uint(__uint_as_float(0x4B000000u | b) - 8388736.0f) >> 16);
+    }
+}
+
+}  // namespace f64tc
+
+inline int f64tc_kblocks(int N) { return (N + 15) / 16; }
+
+}  // namespace gbs

@@ -205,6 +205,9 @@ void release_all(gbs_net *net) {
     net_free(net, net->d_sq64);
     net_free(net, net->d_sq32);
     net_free(net, net->d_T64);
+    net_free(net, net->d_Aq);
+    net_free(net, net->d_rowexp);
+    net_free(net, net->d_colexp);
     net_free(net, net->d_A);
     pool_free(net->d_B, net->stream);
     pool_free(net->d_B_alt, net->stream);
@@ -521,6 +524,43 @@ int finish_device_T(gbs_net *net, unsigned long long *d_bad) {
     return GBS_OK;
 }
 
+// The operand of the FP64 GEMM on the tensor cores from d_T64, which is
+// released.  Networks whose squeezing or rows of T lie outside the range of
+// the digits' scales, or whose digits do not fit in memory, keep d_T64 and the
+// SIMT kernel.
+int make_f64tc_operand(gbs_net *net, const std::vector<double2> &sq) {
+    std::vector<int> e;
+    if (!f64tc_column_exponents(sq, e)) return GBS_OK;
+    int rc;
+    unsigned long long *d_bad = nullptr, bad = 0;
+    auto drop = [&] {
+        net_free(net, net->d_Aq);
+        net_free(net, net->d_rowexp);
+        net_free(net, net->d_colexp);
+    };
+    if ((rc = net_alloc(net, &net->d_colexp, (size_t)net->N, "mode exponents")) ||
+        (rc = net_alloc(net, &net->d_rowexp, (size_t)net->mtiles * 128, "row exponents")) ||
+        (rc = net_alloc(net, &net->d_Aq, f64tc_A_bytes(net->N, net->mtiles), "digits of T")) ||
+        (rc = net_alloc(net, &d_bad, (size_t)1, "range check"))) {
+        drop();
+        return rc == GBS_ENOMEM ? GBS_OK : rc;
+    }
+    if (cudaMemcpyAsync(net->d_colexp, e.data(), sizeof(int) * net->N, cudaMemcpyHostToDevice,
+                        net->stream) != cudaSuccess ||
+        cudaMemsetAsync(d_bad, 0, sizeof(bad), net->stream) != cudaSuccess)
+        rc = set_error(GBS_ECUDA, "upload of the mode exponents failed");
+    if (!rc) rc = launch_f64tc_split_T(net, d_bad);
+    if (!rc && (cudaMemcpyAsync(&bad, d_bad, sizeof(bad), cudaMemcpyDeviceToHost, net->stream) !=
+                    cudaSuccess ||
+                cudaStreamSynchronize(net->stream) != cudaSuccess))
+        rc = set_error(GBS_ECUDA, "digits of T failed");
+    net_free(net, d_bad);
+    if (rc) return rc;
+    if (bad) drop();
+    else net_free(net, net->d_T64);
+    return GBS_OK;
+}
+
 // Shared by gbs_make_network (T in host memory) and gbs_make_network_device.
 int make_network(int N, int M, const double *T, bool T_device, const double *r, int precision,
                  void *stream, gbs_net_t *out) {
@@ -634,6 +674,8 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
         rc = finish_device_T(net, d_bad);
         net_free(net, d_bad);
         if (rc) return fail(rc);
+        if (precision == GBS_FP64 && N >= kF64tcMinN && (rc = make_f64tc_operand(net, sq64)))
+            return fail(rc);
     } else {
         // A = [Re T_i.; Im T_i.] rows interleaved per output mode, T rounded to
         // FP32 and split into BF16 planes T = T0 + T1 + T2, each plane
@@ -664,7 +706,8 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
     // chunk workspace
     net->chunk = pick_chunk(net);
     if (simt_precision(precision)) {
-        net->B_bytes = (size_t)net->chunk * 2 * N * sizeof(double);
+        net->B_bytes = net->d_Aq ? f64tc_B_bytes(N, net->chunk)
+                                 : (size_t)net->chunk * 2 * N * sizeof(double);
     } else {
         const int64_t tiles = (net->chunk + kTcTileSamples - 1) / kTcTileSamples;
         net->B_bytes = (size_t)net->planesB * tiles * 256 * net->ldK * sizeof(__nv_bfloat16);

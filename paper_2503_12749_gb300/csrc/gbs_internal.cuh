@@ -45,6 +45,12 @@ constexpr double kSkipLog = 41.58883083359672;    // 60 * ln 2
 constexpr double kSkipLogDf = 32.57791748631743;  // 47 * ln 2
 constexpr int kFp64TileModes = 64;              // output modes per FP64 GEMM tile
 constexpr int kFp64TileSamples = 32;            // samples per FP64 GEMM tile
+// Input modes from which the FP64 GEMM runs as digit products on the tensor
+// cores (k_gemm_f64tc.cu): one whole K step.  It is the faster one at every
+// size (N = M = 16, 16384 trajectories: 0.054 against 0.150 ms), but its
+// error grows as sqrt(N) against the FMA chain's N, and below about 10 modes
+// the chain's is the smaller.
+constexpr int kF64tcMinN = 16;
 constexpr int kTcTileModes = 64;                // output modes per tcgen05 tile (128 A rows)
 constexpr int kTcTileSamples = 128;             // samples per tcgen05 tile (256 B rows)
 constexpr int kTcBlockK = 64;                   // K elements per pipeline stage (128 B of bf16)
@@ -155,6 +161,13 @@ struct gbs_net {
     // FP64 network operand: [M][2][N], row (i,0) = Re T_i., (i,1) = Im T_i.
     double *d_T64 = nullptr;
 
+    // GBS_FP64 on the tensor cores (k_gemm_f64tc.cu): the network operand as
+    // digit tiles, its row exponents (mtiles * 128), the input modes'
+    // exponents (N); d_Aq set = this network runs that path (its sample
+    // operand d_B then holds digit tiles and d_T64 is not kept)
+    uint8_t *d_Aq = nullptr;
+    int *d_rowexp = nullptr, *d_colexp = nullptr;
+
     // BF16 split operands (GBS_BF16X3 / X6): planes of A = [Re T; Im T] rows
     // interleaved per mode, K-blocked: [planes][ldK / 32][rowsA][32] bf16,
     // ldK = N rounded up to a multiple of 32 (the sample operand likewise)
@@ -251,6 +264,15 @@ SampleJob sample_job_bf16(gbs_net *net, void *B, double *n, uint64_t seed, uint6
 
 // Propagation GEMM with the fused occupation epilogue -> nS_part[mtiles][chunk].
 int launch_gemm_fp64(gbs_net *net, int64_t count, OccOut64 occ = OccOut64());
+// The FP64 GEMM on the tensor cores.  Exponents of the input modes from the
+// sampler coefficients (false: outside the range the digits are used for);
+// digit tiles of T from d_T64 (*d_bad counts rows outside the range); bytes
+// of the two operands.
+bool f64tc_column_exponents(const std::vector<double2> &sq, std::vector<int> &e);
+int launch_f64tc_split_T(gbs_net *net, unsigned long long *d_bad);
+int launch_gemm_f64tc(gbs_net *net, int64_t count, OccOut64 occ);
+size_t f64tc_A_bytes(int N, int mtiles);
+size_t f64tc_B_bytes(int N, int64_t chunk);
 int tc_plan_create(gbs_net *net);
 void tc_plan_destroy(gbs_net *net);
 int launch_gemm_tc(gbs_net *net, int64_t count, OccOut occ = OccOut());

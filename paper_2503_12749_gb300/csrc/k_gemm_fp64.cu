@@ -187,6 +187,7 @@ void launch_dfma_rate(bool outer, int blocks, int threads, cudaStream_t st, doub
 int launch_gemm_fp64(gbs_net *net, int64_t count, OccOut64 occ) {
     if (count <= 0) return GBS_OK;
     if (occ.p && occ.ld < count) return set_error(GBS_EINVAL, "occupation ld < count");
+    if (net->d_Aq) return launch_gemm_f64tc(net, count, occ);
     const int64_t sblocks = (count + TS - 1) / TS;
     if (sblocks > 0x7fffffff) return set_error(GBS_EINVAL, "chunk too large");
     dim3 grid((unsigned)sblocks, (unsigned)net->mtiles);

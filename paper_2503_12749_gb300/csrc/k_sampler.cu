@@ -21,6 +21,7 @@
 // device code (sampler_dev.cuh) also runs in the spare warps of the
 // 3-product GEMM, which sample the next chunk.
 #include "gbs_internal.cuh"
+#include "f64tc.cuh"
 #include "sampler_dev.cuh"
 
 namespace gbs {
@@ -76,6 +77,72 @@ __global__ void k_sample_fp64(const double2 *__restrict__ sq, int N, uint64_t se
 }
 
 // ---------------------------------------------------------------------------
+// FP64 path on the tensor cores: the digit tiles of f64tc.cuh.  A block holds
+// 8 trajectories (one core matrix) and its 4 warps take 16 groups of 8
+// consecutive modes per pass, a lane one group of one trajectory: it stores 16
+// bytes per digit, the 8 lanes of a group one 128-byte core matrix.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(128) k_sample_f64tc(const double2 *__restrict__ sq,
+                                                      const int *__restrict__ col_exp, int N,
+                                                      int KB, uint64_t seed, uint64_t e0,
+                                                      int64_t count, uint8_t *__restrict__ B,
+                                                      double *__restrict__ n_out) {
+    using namespace f64tc;
+    __shared__ double s_n[4][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 8 + (lane & 7);
+    const uint64_t e = e0 + (uint64_t)i;
+    const int row = (int)(i & 15);
+    uint8_t *tile = B + (size_t)(i / kTrajTile) * KB * kBStage + ((i >> 4) & 1) * kBSub;
+    double part = 0.0;
+    if (i < count)
+        for (int oct = warp * 4 + (lane >> 3); oct < 2 * KB; oct += 16) {
+            uint32_t da[kDigits][4], db[kDigits][4];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const int j = oct * 8 + t;
+                uint16_t pa[kDigits] = {}, pb[kDigits] = {};
+                if (j < N) {
+                    double w1, w2;
+                    normals_fp64(seed, e, (uint32_t)j, w1, w2);
+                    const double2 q = sq[j];
+                    const double a = q.x * w1 + q.y * w2;
+                    const double b = q.x * w1 - q.y * w2;
+                    const int s = 55 - col_exp[j];
+                    digits_bf16(to_fixed(a, s), pa);
+                    digits_bf16(to_fixed(b, s), pb);
+                    part += a * b;
+                }
+#pragma unroll
+                for (int q = 0; q < kDigits; ++q) {
+                    if (t & 1) {
+                        da[q][t >> 1] |= (uint32_t)pa[q] << 16;
+                        db[q][t >> 1] |= (uint32_t)pb[q] << 16;
+                    } else {
+                        da[q][t >> 1] = pa[q];
+                        db[q][t >> 1] = pb[q];
+                    }
+                }
+            }
+            uint8_t *p = tile + (size_t)(oct >> 1) * kBStage;
+            const int k = (oct & 1) * 8;
+#pragma unroll
+            for (int q = 0; q < kDigits; ++q) {
+                *reinterpret_cast<uint4 *>(p + q * kBSlice + core_offset(row, k)) =
+                    make_uint4(da[q][0], da[q][1], da[q][2], da[q][3]);
+                *reinterpret_cast<uint4 *>(p + q * kBSlice + core_offset(16 + row, k)) =
+                    make_uint4(db[q][0], db[q][1], db[q][2], db[q][3]);
+            }
+        }
+    part += __shfl_xor_sync(0xffffffffu, part, 8);
+    part += __shfl_xor_sync(0xffffffffu, part, 16);
+    if (lane < 8) s_n[warp][lane] = part;
+    __syncthreads();
+    if (threadIdx.x < 8 && i < count)
+        n_out[i] = (s_n[0][lane] + s_n[1][lane]) + (s_n[2][lane] + s_n[3][lane]);
+}
+
+// ---------------------------------------------------------------------------
 // BF16 split path: FP32 arithmetic; each lane handles 4 consecutive modes.
 // ---------------------------------------------------------------------------
 template <bool kSfu>
@@ -100,6 +167,13 @@ int grid_for_warps(gbs_net *net, int64_t warps_needed, int threads) {
 int launch_sample_fp64(gbs_net *net, uint64_t seed, uint64_t e0, int64_t count) {
     net->pre_valid = false;  // the operands are overwritten
     if (count <= 0) return GBS_OK;
+    if (net->d_Aq) {
+        k_sample_f64tc<<<(unsigned)((count + 7) / 8), 128, 0, net->stream>>>(
+            net->d_sq64, net->d_colexp, net->N, f64tc_kblocks(net->N), seed, e0, count,
+            static_cast<uint8_t *>(net->d_B), net->d_n);
+        GBS_LAUNCH_CHECK();
+        return GBS_OK;
+    }
     const int threads = 256;
     k_sample_fp64<<<grid_for_warps(net, count, threads), threads, 0, net->stream>>>(
         net->d_sq64, net->N, seed, e0, count, static_cast<double *>(net->d_B), net->d_n);
