@@ -17,18 +17,20 @@
 // e^{-l1} term) outside which each term is provably smaller than that,
 // using |sin theta| <= sqrt(2 (1 - cos theta)).
 //
-// Work split (FP64 kernel): one thread per k, one block per (256
-// consecutive k, sub-ensemble r); each thread loops over the sub-ensemble's
-// trajectories of the chunk in increasing order and adds its sums to
-// acc[est][r][k], so every sum is formed in a fixed order (bitwise
-// reproducible for a fixed chunking).  The double-float kernel gives each
-// lane the mirror pair k, K1 - k and splits the trajectories over 8
-// half-warps (see k_gf_df).  Trajectory e belongs to sub-ensemble e mod n_sub.
+// Work split: each lane holds the mirror pair k, K1 - k; half-warps (and, in
+// the FP64 kernel, the blocks of a cluster) split a sub-ensemble's
+// trajectories and their sums are combined in a fixed order, so every run is
+// bitwise reproducible for a fixed chunking.  Trajectory e belongs to
+// sub-ensemble e mod n_sub.
 #include "gbs_internal.cuh"
 #include "dfloat.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
+
+namespace cg = cooperative_groups;
 
 namespace gbs {
 namespace {
@@ -145,90 +147,317 @@ __device__ __forceinline__ int dist_pi(int k, int K1) {
     return d < 0 ? -d : d;
 }
 
-// FP64 evaluation (GBS_FP64).
-__global__ void __launch_bounds__(256) k_gf_fp64(const double *__restrict__ n_in,
-                                                 const double2 *__restrict__ nS_in,
-                                                 const Window *__restrict__ win_in,
-                                                 int64_t count, uint64_t e0, int n_sub, int K1,
-                                                 const double2 *__restrict__ tw,
-                                                 double2 *__restrict__ acc,
-                                                 int64_t *__restrict__ counts) {
-    __shared__ double s_x[256], s_y[256], s_c1[256], s_c2[256], s_inv[256];
-    __shared__ int s_w1[256], s_w2[256];
-
-    const int r = blockIdx.y;
-    const int kb0 = blockIdx.x * 256;
-    const int kb1 = min(kb0 + 256, K1);
-    const int k = kb0 + threadIdx.x;
-    const bool kvalid = k < K1;
-    const int d0 = kvalid ? dist0(k, K1) : 0x3fffffff;
-    const int dpi = kvalid ? dist_pi(k, K1) : 0x3fffffff;
-    // block-wide minimum distances (for tile skipping)
-    const int bd0 = min(dist0(kb0, K1), dist0(kb1 - 1, K1));
+// Pair slots of the union window: slot s holds k = s and K1 - s for
+// s = 0..W1 (around theta = 0), then k = K1/2 + s and K1/2 - s for
+// s = 0..W2 (around theta = pi); when the two windows cover the circle,
+// s = 0..K1/2.  k = 0 and k = K1/2 pair with themselves.
+__device__ __forceinline__ int pair_slot_count(int K1, int W1, int W2, bool &whole) {
     const int half = K1 >> 1;
-    const int bdpi = (half >= kb0 && half < kb1) ? 0 : min(dist_pi(kb0, K1), dist_pi(kb1 - 1, K1));
+    const int n1 = W1 >= half ? K1 : 2 * W1 + 1;
+    const int n2 = W2 < 0 ? 0 : (W2 >= half ? K1 : 2 * W2 + 1);
+    whole = n1 + n2 >= K1;
+    if (whole) return half + 1;
+    return (W1 < 0 ? 0 : W1 + 1) + (W2 < 0 ? 0 : W2 + 1);
+}
 
+// (k, K1 - k) of pair slot i (whole: the windows cover the circle), or
+// kp = -1 past the end.
+__device__ __forceinline__ void pair_slot_to_k(int i, int K1, int W1, int W2, bool whole, int &kp,
+                                               int &km) {
+    const int half = K1 >> 1;
+    kp = km = -1;
+    if (whole) {
+        if (i <= half) {
+            kp = i;
+            km = (K1 - i) & (K1 - 1);
+        }
+        return;
+    }
+    const int p1 = W1 < 0 ? 0 : W1 + 1;
+    const int p2 = W2 < 0 ? 0 : W2 + 1;
+    if (i < p1) {
+        kp = i;
+        km = (K1 - i) & (K1 - 1);
+    } else if (i < p1 + p2) {
+        kp = half + (i - p1);
+        km = half - (i - p1);
+    }
+}
+
+
+// ---------------------------------------------------------------------------
+// FP64 evaluation (GBS_FP64, GBS_FP32).
+//
+// Bound by the FP64 pipe (2 lanes per SM and clock), so the kernel is built to
+// issue few FP64 instructions per term: exp and sin/cos by tables (2^(j/64),
+// 256 points of the circle) and short Taylor polynomials of the reduced
+// argument, table indices taken from the low bits of a magic-number addition
+// (Tang, "Table-driven implementation of the exponential function in IEEE
+// floating-point arithmetic", ACM TOMS 15, 1989; the same for sin and cos by
+// angle addition): about 33 FP64 instructions per complex exponential, against
+// about 80 for exp and sincos.  The lane holds the mirror pair k, K1 - k (see
+// "Mirror pairs" below): for n_S real up to rounding one complex exponential
+// serves both, through the moment sums S_j = sum E y^j, j = 0..2.  The
+// trajectories of a sub-ensemble are split over half-warps and the blocks of a
+// cluster: one thread per k walking all of them left a 64-point circle to 1024
+// threads.  Measured (ms, before -> now): N = 16, K1 = 64, 16384 trajectories in 16
+// sub-ensembles 2.39 -> 0.16; N = 1000, K1 = 4096, 32768 in 100 3.60 -> 0.61
+// (5.3e6 pairs, 0.56 of the FP64 pipe); a 615 x 700 network with complex n_S,
+// K1 = 2048, 20001 in 37 2.63 -> 0.74.
+// ---------------------------------------------------------------------------
+struct Gf64Tables {         // each value as a double and its rounding error
+    double2 exp2[64];         // 2^(j/64)
+    double2 sn[256], cs[256]; // sin, cos of 2 pi j / 256
+};
+
+constexpr double kMagic = 6755399441055744.0;  // 1.5 2^52
+
+// e^a for a in [-700, 700] (below, e^-700): one rounding above the reduced
+// argument's, the table's own rounding error added back.
+__device__ __forceinline__ double exp_tab64(double a, const Gf64Tables &T) {
+    if (a > 700.0) return exp(a);
+    a = a < -700.0 ? -700.0 : a;
+    const double t = fma(a, 0x1.71547652b82fep+6, kMagic);  // 64 / ln 2
+    const int n = __double2loint(t);
+    const double nf = t - kMagic;
+    // ln 2 / 64 in a 36-bit piece (products with |n| < 2^17 exact) and the rest
+    double r = fma(nf, -0x1.62e42fefap-7, a);
+    r = fma(nf, -0x1.cf79abc9e3b3ap-46, r);
+    double p = fma(r, 1.0 / 720.0, 1.0 / 120.0);
+    p = fma(p, r, 1.0 / 24.0);
+    p = fma(p, r, 1.0 / 6.0);
+    p = fma(p, r, 0.5);
+    p = fma(p, r * r, r);  // e^r - 1; r^7 / 5040 < 2^-64
+    const double2 s = T.exp2[n & 63];
+    const double v = s.x + fma(s.x, p, s.y);
+    return __hiloint2double(__double2hiint(v) + ((n >> 6) << 20), __double2loint(v));
+}
+
+// (sin a, cos a) for |a| < 2.5e4 (table as above), else sincos.
+__device__ __forceinline__ void sincos_tab64(double a, const Gf64Tables &T, double &sn, double &cs) {
+    if (!(fabs(a) < 2.5e4)) {
+        sincos(a, &sn, &cs);
+        return;
+    }
+    const double t = fma(a, 0x1.45f306dc9c883p+5, kMagic);  // 256 / (2 pi)
+    const int n = __double2loint(t);
+    const double nf = t - kMagic;
+    // 2 pi / 256 in a 33-bit piece (products with |n| < 2^20 exact) and the rest
+    double r = fma(nf, -0x1.921fb544p-6, a);
+    r = fma(nf, -0x1.0b4611a626331p-40, r);
+    const double q = r * r;
+    double ps = fma(q, -1.0 / 5040.0, 1.0 / 120.0);
+    ps = fma(ps, q, -1.0 / 6.0);
+    const double s = fma(ps, r * q, r);  // sin r; r^9 / 9! < 2^-69 r
+    double pc = fma(q, -1.0 / 720.0, 1.0 / 24.0);
+    pc = fma(pc, q, -0.5) * q;           // cos r - 1; r^8 / 8! < 2^-65
+    const double2 S = T.sn[n & 255], C = T.cs[n & 255];
+    sn = S.x + fma(C.x, s, fma(S.x, pc, S.y));
+    cs = C.x + fma(-S.x, s, fma(C.x, pc, C.y));
+}
+
+constexpr int kG64Slots = 16;   // mirror pairs per block, the lanes of each half-warp
+constexpr int kG64Groups = 8;   // half-warps per block, splitting the trajectories
+constexpr int kG64Per = 16;     // trajectories per half-warp and tile
+constexpr int kG64MaxCluster = 8;
+// |y| |sin|, |y| |cos - 1| up to here go through the moment sums: then
+// |omega| <= 2^-17.5 and omega^3 / 6 < 2^-55 is left out
+constexpr double kG64Mirror = 0x1p-18;
+
+struct Gf64Rec {
+    double x, y, c1, c2, inv;
+    int w1, w2;
+};
+
+struct Gf64Shared {
+    Gf64Tables tab;
+    Gf64Rec rec[kG64Groups][kG64Per];
+    // general terms of each lane: [k, K1 - k][matrix-P re, im, +P re, im]
+    double gen[2][4][kG64Slots * kG64Groups];
+    // the block's sums, read by the cluster's first block
+    double out[2][4][kG64Slots];
+};
+
+// One term by the general formulas at (l1, ph) = (z - 1) n_S.
+__device__ __forceinline__ void gf64_term(double l1, double ph, bool in1, bool in2,
+                                          const Gf64Rec &g, const Gf64Tables &T, double *f) {
+    constexpr int ld = kG64Slots * kG64Groups;
+    double sp, cp;
+    sincos_tab64(ph, T, sp, cp);
+    double e1 = 0.0, e2 = 0.0;
+    if (in1) {
+        e1 = exp_tab64(l1 + g.c1, T);
+        const double gp = (g.c1 == 0.0) ? e1 : exp_tab64(l1, T);
+        f[2 * ld] += gp * cp;
+        f[3 * ld] += gp * sp;
+    }
+    if (in2) e2 = exp_tab64(g.c2 - l1, T);
+    f[0] += (e1 + e2) * cp * g.inv;
+    f[ld] += (e1 - e2) * sp * g.inv;
+}
+
+// S0 + w^2 S2 / 2 +- w S1 added to the lane's sums at k and (conjugated) K1 - k.
+struct Gf64Moments {
+    double r0, i0, r1, i1, r2, i2;
+};
+__device__ __forceinline__ void gf64_finish(const Gf64Moments &m, double wr, double wi, double *fk,
+                                            double *fm) {
+    constexpr int ld = kG64Slots * kG64Groups;
+    const double vr = 0.5 * (wr * wr - wi * wi), vi = wr * wi;  // w^2 / 2
+    const double xr = m.r0 + (vr * m.r2 - vi * m.i2), xi = m.i0 + (vr * m.i2 + vi * m.r2);
+    const double zr = wr * m.r1 - wi * m.i1, zi = wr * m.i1 + wi * m.r1;
+    fk[0] += xr + zr;
+    fk[ld] += xi + zi;
+    fm[0] += xr - zr;
+    fm[ld] -= xi - zi;
+}
+
+// Grid: x = (sub-ensemble, block of the cluster), y = 16 pair slots from k = 0
+// outwards (heaviest first).  The blocks of a cluster and their half-warps
+// split the sub-ensemble's trajectories (trajectory q to half-warp q mod
+// (8 C)); the sums are combined in a fixed order, within the block through
+// shared memory and across the cluster through distributed shared memory.
+__global__ void __launch_bounds__(kG64Slots *kG64Groups)
+    k_gf_fp64(const double *__restrict__ n_in, const double2 *__restrict__ nS_in,
+              const Window *__restrict__ win_in, const int *__restrict__ wmax, int64_t count,
+              uint64_t e0, int n_sub, int K1, const double2 *__restrict__ tw, const Gf64Tables tabs,
+              double2 *__restrict__ acc, int64_t *__restrict__ counts) {
+    __shared__ Gf64Shared sh;
+    constexpr int ld = kG64Slots * kG64Groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int C = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
+    const int r = blockIdx.x / C;
+    bool whole;
+    const int nslots = pair_slot_count(K1, wmax[0], wmax[1], whole);
     const int64_t first = (int64_t)(((uint64_t)r + (uint64_t)n_sub - e0 % (uint64_t)n_sub) %
                                     (uint64_t)n_sub);
     const int64_t cnt_r = first < count ? (count - 1 - first) / n_sub + 1 : 0;
+    if (blockIdx.y == 0 && crank == 0 && threadIdx.x == 0) counts[r] += cnt_r;
+    if ((int)blockIdx.y * kG64Slots >= nslots) return;  // the whole cluster
+    const int slot = threadIdx.x & (kG64Slots - 1), grp = threadIdx.x / kG64Slots;
+    int kp, km;
+    pair_slot_to_k(blockIdx.y * kG64Slots + slot, K1, wmax[0], wmax[1], whole, kp, km);
+    const bool kvalid = kp >= 0, self = kp == km;
+    const int d0 = kvalid ? dist0(kp, K1) : 0x3fffffff;
+    const int dpi = kvalid ? dist_pi(kp, K1) : 0x3fffffff;
+    if (threadIdx.x < 64) sh.tab.exp2[threadIdx.x] = tabs.exp2[threadIdx.x];
+    for (int t = threadIdx.x; t < 256; t += ld) {
+        sh.tab.sn[t] = tabs.sn[t];
+        sh.tab.cs[t] = tabs.cs[t];
+    }
+    double *fk = &sh.gen[0][0][threadIdx.x], *fm = &sh.gen[1][0][threadIdx.x];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) fk[c * ld] = fm[c * ld] = 0.0;
+    __syncthreads();
 
-    double2 t = kvalid ? tw[k] : make_double2(0.0, 0.0);
+    const double2 t = kvalid ? tw[kp] : make_double2(0.0, 0.0);
     const double cm1 = t.x, sn = t.y;
-    double am_re = 0.0, am_im = 0.0, ap_re = 0.0, ap_im = 0.0;
+    const double ymul = fmax(fabs(sn), fabs(cm1));
+    Gf64Moments both = {}, mp = {}, pp = {};  // common terms; matrix-P's, +P's own
+    const int parts = kG64Groups * C, part = crank * kG64Groups + grp;
+    const unsigned hmask = 0xffffu << (threadIdx.x & 16);
 
-    for (int64_t base = 0; base < cnt_r; base += 256) {
-        const int64_t q = base + threadIdx.x;
-        int hit = 0;
-        if (q < cnt_r) {
-            const int64_t i = first + q * n_sub;
-            const double nn = n_in[i];
-            const double2 s = nS_in[i];
-            const Window w = win_in[i];
-            s_x[threadIdx.x] = s.x;
-            s_y[threadIdx.x] = s.y;
-            s_c1[threadIdx.x] = fmin(0.0, 2.0 * nn);
-            s_c2[threadIdx.x] = -2.0 * fmax(nn, 0.0);
-            s_inv[threadIdx.x] = 1.0 / (1.0 + exp(-2.0 * fabs(nn)));
-            s_w1[threadIdx.x] = w.w1;
-            s_w2[threadIdx.x] = w.w2;
-            hit = (bd0 <= w.w1) || (bdpi <= w.w2);
-        }
-        if (!__syncthreads_or(hit)) continue;
-        const int ntile = (cnt_r - base) < 256 ? (int)(cnt_r - base) : 256;
-        if (kvalid) {
-            for (int j = 0; j < ntile; ++j) {
-                const bool in1 = d0 <= s_w1[j];
-                const bool in2 = dpi <= s_w2[j];
-                if (!(in1 || in2)) continue;
-                const double x = s_x[j], y = s_y[j];
-                const double l1 = cm1 * x - sn * y;
-                const double ph = sn * x + cm1 * y;
-                double sp, cp;
-                sincos(ph, &sp, &cp);
-                double e1 = 0.0, e2 = 0.0;
-                if (in1) {
-                    const double c1 = s_c1[j];
-                    e1 = exp(l1 + c1);
-                    const double gp = (c1 == 0.0) ? e1 : exp(l1);
-                    ap_re += gp * cp;
-                    ap_im += gp * sp;
-                }
-                if (in2) e2 = exp(-l1 + s_c2[j]);
-                const double inv = s_inv[j];
-                am_re += (e1 + e2) * cp * inv;
-                am_im += (e1 - e2) * sp * inv;
+    for (int64_t base = part; base < cnt_r; base += (int64_t)parts * kG64Per) {
+        __syncwarp(hmask);
+        {
+            const int64_t q = base + (int64_t)slot * parts;
+            if (q < cnt_r) {
+                const int64_t i = first + q * n_sub;
+                const double nn = n_in[i], an = fabs(nn);
+                const double2 s = nS_in[i];
+                const Window w = win_in[i];
+                Gf64Rec g;
+                g.x = s.x;
+                g.y = s.y;
+                g.c1 = fmin(0.0, 2.0 * nn);
+                g.c2 = -2.0 * fmax(nn, 0.0);
+                g.inv = an > 20.0 ? 1.0 : 1.0 / (1.0 + exp(-2.0 * an));  // e^-40 < 2^-54
+                g.w1 = w.w1;
+                g.w2 = w.w2;
+                sh.rec[grp][slot] = g;
             }
         }
-        __syncthreads();
+        __syncwarp(hmask);
+        const int64_t left = (cnt_r - base + parts - 1) / parts;
+        const int nt = left < kG64Per ? (int)left : kG64Per;
+        if (!kvalid) continue;
+        for (int j = 0; j < nt; ++j) {
+            const Gf64Rec &g = sh.rec[grp][j];
+            const bool in1 = d0 <= g.w1, in2 = dpi <= g.w2;
+            if (!(in1 || in2)) continue;
+            const double x = g.x, y = g.y;
+            const double a = cm1 * x, c = sn * x;
+            if (g.c1 == 0.0 && fabs(y) * ymul <= kG64Mirror) {
+                // n >= 0: e^{l1} serves both estimators
+                double sp, cp;
+                sincos_tab64(c, sh.tab, sp, cp);
+                const double e1 = in1 ? exp_tab64(a, sh.tab) : 0.0;
+                const double re = e1 * cp, im = e1 * sp;
+                if (!in2 && g.inv == 1.0) {
+                    both.r0 += re;
+                    both.i0 += im;
+                    both.r1 = fma(re, y, both.r1);
+                    both.i1 = fma(im, y, both.i1);
+                    const double y2 = y * y;
+                    both.r2 = fma(re, y2, both.r2);
+                    both.i2 = fma(im, y2, both.i2);
+                } else {
+                    // matrix-P: inv (e^{a} e^{ic} e^{omega} + e^{-a + c2} e^{-ic} e^{-omega})
+                    const double e2 = in2 ? exp_tab64(g.c2 - a, sh.tab) : 0.0;
+                    const double cv = cp * g.inv, sv = sp * g.inv;
+                    const double ep = e1 + e2, em = e1 - e2;
+                    const double er = ep * cv, ei = em * sv;  // even moments
+                    const double orr = em * cv, oi = ep * sv;  // odd moments
+                    const double y2 = y * y;
+                    mp.r0 += er;
+                    mp.i0 += ei;
+                    mp.r1 = fma(orr, y, mp.r1);
+                    mp.i1 = fma(oi, y, mp.i1);
+                    mp.r2 = fma(er, y2, mp.r2);
+                    mp.i2 = fma(ei, y2, mp.i2);
+                    if (in1) {
+                        pp.r0 += re;
+                        pp.i0 += im;
+                        pp.r1 = fma(re, y, pp.r1);
+                        pp.i1 = fma(im, y, pp.i1);
+                        pp.r2 = fma(re, y2, pp.r2);
+                        pp.i2 = fma(im, y2, pp.i2);
+                    }
+                }
+                continue;
+            }
+            const double b = sn * y, d = cm1 * y;
+            gf64_term(fma(cm1, x, -b), fma(sn, x, d), in1, in2, g, sh.tab, fk);
+            if (!self) gf64_term(fma(cm1, x, b), fma(-sn, x, d), in1, in2, g, sh.tab, fm);
+        }
     }
-    if (kvalid) {
-        double2 *a0 = acc + (size_t)r * K1 + k;
-        double2 *a1 = acc + ((size_t)n_sub + r) * K1 + k;
-        const double2 o0 = *a0, o1 = *a1;
-        *a0 = make_double2(o0.x + am_re, o0.y + am_im);
-        *a1 = make_double2(o1.x + ap_re, o1.y + ap_im);
+    gf64_finish(both, -sn, cm1, fk, fm);
+    gf64_finish(both, -sn, cm1, fk + 2 * ld, fm + 2 * ld);
+    gf64_finish(mp, -sn, cm1, fk, fm);
+    gf64_finish(pp, -sn, cm1, fk + 2 * ld, fm + 2 * ld);
+    __syncthreads();
+    // 2 sides x 4 sums x 16 slots, one per thread: the half-warps in order
+    {
+        const int side = threadIdx.x >> 6, q = (threadIdx.x >> 4) & 3;
+        double v = 0.0;
+#pragma unroll
+        for (int gi = 0; gi < kG64Groups; ++gi) v += sh.gen[side][q][gi * kG64Slots + slot];
+        sh.out[side][q][slot] = v;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) counts[r] += cnt_r;
+    if (C > 1) cluster.sync();
+    else __syncthreads();
+    if (crank == 0 && kvalid) {
+        const int side = threadIdx.x >> 6, q = (threadIdx.x >> 4) & 3;
+        if (!(side && self)) {
+            double v = 0.0;
+            for (int b = 0; b < C; ++b) v += cluster.map_shared_rank(&sh.out[side][q][slot], b)[0];
+            double *dst = reinterpret_cast<double *>(
+                              acc + ((size_t)(q >> 1) * n_sub + r) * K1 + (side ? km : kp)) +
+                          (q & 1);
+            *dst += v;
+        }
+    }
+    if (C > 1) cluster.sync();  // the other blocks' sums stay readable until here
 }
 
 // Double-float evaluation (BF16 split paths).  Each generating-function
@@ -395,43 +624,6 @@ __device__ __forceinline__ void mirror_finish(const MirrorSums &m, df2 w, df2 &a
     at_mk = df2_add(X, Z);
     at_mk.hi.y = -at_mk.hi.y;
     at_mk.lo.y = -at_mk.lo.y;
-}
-
-// Pair slots of the union window: slot s holds k = s and K1 - s for
-// s = 0..W1 (around theta = 0), then k = K1/2 + s and K1/2 - s for
-// s = 0..W2 (around theta = pi); when the two windows cover the circle,
-// s = 0..K1/2.  k = 0 and k = K1/2 pair with themselves.
-__device__ __forceinline__ int pair_slot_count(int K1, int W1, int W2, bool &whole) {
-    const int half = K1 >> 1;
-    const int n1 = W1 >= half ? K1 : 2 * W1 + 1;
-    const int n2 = W2 < 0 ? 0 : (W2 >= half ? K1 : 2 * W2 + 1);
-    whole = n1 + n2 >= K1;
-    if (whole) return half + 1;
-    return (W1 < 0 ? 0 : W1 + 1) + (W2 < 0 ? 0 : W2 + 1);
-}
-
-// (k, K1 - k) of pair slot i (whole: the windows cover the circle), or
-// kp = -1 past the end.
-__device__ __forceinline__ void pair_slot_to_k(int i, int K1, int W1, int W2, bool whole, int &kp,
-                                               int &km) {
-    const int half = K1 >> 1;
-    kp = km = -1;
-    if (whole) {
-        if (i <= half) {
-            kp = i;
-            km = (K1 - i) & (K1 - 1);
-        }
-        return;
-    }
-    const int p1 = W1 < 0 ? 0 : W1 + 1;
-    const int p2 = W2 < 0 ? 0 : W2 + 1;
-    if (i < p1) {
-        kp = i;
-        km = (K1 - i) & (K1 - 1);
-    } else if (i < p1 + p2) {
-        kp = half + (i - p1);
-        km = half - (i - p1);
-    }
 }
 
 constexpr int kGfSlots = 16;   // pair slots per block (the lanes of each half-warp)
@@ -736,6 +928,32 @@ __global__ void __launch_bounds__(kGfSlots * kGfGroups, GBS_GF_MINBLOCKS)
 
 }  // namespace
 
+namespace {
+
+Gf64Tables make_gf64_tables() {
+    Gf64Tables T;
+    // long double exceeds double on both host architectures; elsewhere the
+    // rounding errors come out as zero and the tables as plain doubles
+    auto pair = [](long double v) {
+        const double hi = (double)v;
+        return make_double2(hi, (double)(v - (long double)hi));
+    };
+    for (int j = 0; j < 64; ++j) T.exp2[j] = pair(std::exp2((long double)j / 64.0L));
+    const long double pi = 3.141592653589793238462643383279502884L;
+    for (int j = 0; j < 256; ++j) {
+        // first-octant arguments, so that the axes come out exactly
+        const int q = j >> 6, m = j & 63;
+        const long double sm = m <= 32 ? std::sin(pi * m / 128.0L) : std::cos(pi * (64 - m) / 128.0L);
+        const long double cm = m <= 32 ? std::cos(pi * m / 128.0L) : std::sin(pi * (64 - m) / 128.0L);
+        const long double sv = (q & 1) ? cm : sm, cv = (q & 1) ? sm : cm;
+        T.sn[j] = pair(q >= 2 ? -sv : sv);
+        T.cs[j] = pair(q == 1 || q == 2 ? -cv : cv);
+    }
+    return T;
+}
+
+}  // namespace
+
 // Float pieces of ln 2 and pi/2 for exact Cody-Waite products (12
 // significant bits each except the last), split from the constants'
 // decimal expansions at 80 digits; factorial reciprocals as double-float.
@@ -814,11 +1032,31 @@ int launch_finalize(gbs_net *net, int64_t count) {
 
 int launch_gf(gbs_net *net, uint64_t e0, int64_t count) {
     if (count <= 0) return GBS_OK;
-    dim3 grid((unsigned)((net->K1 + 255) / 256), (unsigned)net->n_sub);
     if (simt_precision(net->precision)) {
-        k_gf_fp64<<<grid, 256, 0, net->stream>>>(net->d_n, net->d_nS, net->d_win, count, e0,
-                                                   net->n_sub, net->K1, net->d_tw, net->d_acc,
-                                                   net->d_counts);
+        static const Gf64Tables T = make_gf64_tables();
+        // Blocks per sub-ensemble: enough for 8 blocks per SM with up to 11
+        // blocks of pair slots (what the windows of a 1000-mode network
+        // leave), each half-warp keeping at least 16 trajectories
+        const int slots = (net->K1 / 2 + 1 + kG64Slots - 1) / kG64Slots;
+        const int64_t per = count / net->n_sub / kG64Groups;
+        int C = 1;
+        while (C < kG64MaxCluster && per >= 32 * C &&
+               (int64_t)net->n_sub * C * std::min(slots, 11) < 8 * (int64_t)net->sm_count)
+            C *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(net->n_sub * C), (unsigned)slots);
+        cfg.blockDim = dim3(kG64Slots * kG64Groups);
+        cfg.stream = net->stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        GBS_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_gf_fp64, (const double *)net->d_n,
+                                        (const double2 *)net->d_nS, (const Window *)net->d_win,
+                                        (const int *)net->d_wmax, count, e0, net->n_sub, net->K1,
+                                        (const double2 *)net->d_tw, T, net->d_acc, net->d_counts));
     } else {
         static const DfConsts K = make_df_consts();
         dim3 g2((unsigned)net->n_sub, (unsigned)((net->K1 / 2 + 1 + kGfSlots - 1) / kGfSlots));
