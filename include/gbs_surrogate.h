@@ -103,8 +103,7 @@ int gbs_mlp_gradients(gbs_mlp_t mlp, const float *X_dev, const float *T_dev, int
 
 /*
  * gbs_mlp_train -- `steps` full-batch Adam steps on (X_dev, T_dev):
- * forward, loss, backward and update per step, captured once as a CUDA
- * graph and replayed.  lr: host, `steps` learning rates (step i uses lr[i]).
+ * forward, loss, backward and update per step.  lr: host, `steps` learning rates (step i uses lr[i]).
  * loss_hist: host, receives the loss before each step (may be NULL).
  * Synchronises.  Errors: EINVAL, ECUDA, ETIMEOUT.
  */

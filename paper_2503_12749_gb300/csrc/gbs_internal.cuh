@@ -429,11 +429,11 @@ void count_samples(gbs_net *net, uint64_t first, int64_t E);
 void prof_mark(gbs_net *net, int phase, int launches_if_stop, bool start);
 
 // Tensor map of a row-major BF16 array (rows x inner elements, row pitch
-// row_bytes) read in boxes of box_inner x box_rows with the 64-byte swizzle
-// (box_inner = 32 elements = one 64-byte row).  Out-of-range box rows read as
-// zeros.
+// row_bytes) read in boxes of box_inner x box_rows with a swizzle of the box's
+// row (64 bytes for box_inner = 32, 128 for 64).  Box elements out of range read
+// as zeros.
 int encode_2d(CUtensorMap *map, void *base, uint64_t inner, uint64_t rows, uint64_t row_bytes,
-              uint32_t box_inner, uint32_t box_rows);
+              uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle);
 
 // Device properties helper.
 bool device_has_tcgen05(int device);
