@@ -850,16 +850,29 @@ int check_batch(gbs_mlp *m, int batch) {
     return GBS_OK;
 }
 
-// packed (user) index <-> master (padded) index
-template <typename F>
-void for_each_param(const gbs_mlp *m, F f) {
-    int64_t u = 0;
-    for (int l = 0; l < m->L; ++l) {
-        const int kin = l == 0 ? m->in_dim : m->width;
-        for (int n = 0; n < m->lay.n_out[l]; ++n)
-            for (int k = 0; k < kin; ++k) f(u++, m->lay.off_W[l] + (int64_t)n * m->lay.k_pad[l] + k);
-        for (int n = 0; n < m->lay.n_out[l]; ++n) f(u++, m->lay.off_b[l] + n);
-    }
+// Whether every value is finite: the largest magnitude's bit pattern (written
+// to vectorise).
+__attribute__((optimize("O3"))) bool all_finite(const float *v, int64_t n) {
+    const uint32_t *b = reinterpret_cast<const uint32_t *>(v);
+    uint32_t top = 0;
+    for (int64_t i = 0; i < n; ++i) top = std::max(top, b[i] & 0x7fffffffu);
+    return top < 0x7f800000u;
+}
+
+// Packed (user) parameters <-> master layout: the first layer's weights have
+// padded rows, everything after them is the same in both.
+int copy_params(gbs_mlp *m, float *master, float *packed, bool to_device) {
+    const size_t w0 = (size_t)m->width * m->in_dim;
+    const size_t rest = (size_t)(m->nmaster - m->lay.off_b[0]);
+    const cudaMemcpyKind kind = to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
+    const size_t pu = sizeof(float) * m->in_dim, pm = sizeof(float) * kInPad;
+    GBS_CUDA_TRY(cudaMemcpy2DAsync(to_device ? master : packed, to_device ? pm : pu,
+                                   to_device ? packed : master, to_device ? pu : pm, pu,
+                                   (size_t)m->width, kind, m->stream));
+    float *a = master + m->lay.off_b[0], *b = packed + w0;
+    GBS_CUDA_TRY(cudaMemcpyAsync(to_device ? a : b, to_device ? b : a, sizeof(float) * rest, kind,
+                                 m->stream));
+    return GBS_OK;
 }
 
 void destroy(gbs_mlp *m) {
@@ -969,14 +982,15 @@ int gbs_mlp_param_count(gbs_mlp_t m, int64_t *count) {
 
 int gbs_mlp_set_params(gbs_mlp_t m, const float *params) {
     if (!m || !params) return set_error(GBS_EINVAL, "NULL argument");
-    for (int64_t i = 0; i < m->nparams; ++i)
-        if (!std::isfinite(params[i])) return set_error(GBS_EINVAL, "parameter %lld is not finite", (long long)i);
-    std::vector<float> h((size_t)m->nmaster, 0.0f);
-    for_each_param(m, [&](int64_t u, int64_t i) { h[(size_t)i] = params[u]; });
-    GBS_CUDA_TRY(cudaMemcpyAsync(m->master, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice,
-                                 m->stream));
-    GBS_CUDA_TRY(cudaMemsetAsync(m->m1, 0, h.size() * sizeof(float), m->stream));
-    GBS_CUDA_TRY(cudaMemsetAsync(m->m2, 0, h.size() * sizeof(float), m->stream));
+    if (!all_finite(params, m->nparams))
+        for (int64_t i = 0; i < m->nparams; ++i)
+            if (!std::isfinite(params[i])) return set_error(GBS_EINVAL, "parameter %lld is not finite", (long long)i);
+    int rc;
+    const size_t bytes = sizeof(float) * (size_t)m->nmaster;
+    GBS_CUDA_TRY(cudaMemsetAsync(m->master, 0, sizeof(float) * (size_t)m->lay.off_b[0], m->stream));
+    if ((rc = copy_params(m, m->master, const_cast<float *>(params), true))) return rc;
+    GBS_CUDA_TRY(cudaMemsetAsync(m->m1, 0, bytes, m->stream));
+    GBS_CUDA_TRY(cudaMemsetAsync(m->m2, 0, bytes, m->stream));
     GBS_CUDA_TRY(cudaMemsetAsync(m->step, 0, 2 * sizeof(long long), m->stream));
     k_mlp_refresh<<<(unsigned)((m->nmaster + 255) / 256), 256, 0, m->stream>>>(m->lay, m->nmaster,
                                                                                 m->master);
@@ -986,11 +1000,9 @@ int gbs_mlp_set_params(gbs_mlp_t m, const float *params) {
 }
 
 static int copy_packed(gbs_mlp_t m, const float *src_dev, float *dst) {
-    std::vector<float> h((size_t)m->nmaster);
-    GBS_CUDA_TRY(cudaMemcpyAsync(h.data(), src_dev, h.size() * sizeof(float), cudaMemcpyDeviceToHost,
-                                 m->stream));
+    int rc;
+    if ((rc = copy_params(m, const_cast<float *>(src_dev), dst, false))) return rc;
     GBS_CUDA_TRY(cudaStreamSynchronize(m->stream));
-    for_each_param(m, [&](int64_t u, int64_t i) { dst[u] = h[(size_t)i]; });
     return GBS_OK;
 }
 

@@ -13,8 +13,13 @@
 #include "gbs_internal.cuh"
 #include "gbs_surrogate.h"
 
+#include <cooperative_groups.h>
+
+#include <algorithm>
 #include <cmath>
 #include <vector>
+
+namespace cg = cooperative_groups;
 
 namespace gbs {
 namespace {
@@ -58,69 +63,105 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
     return s;
 }
 
-// One block (256 threads) per network.
-__global__ void k_sur_features(const NetIn *__restrict__ nets, const double *__restrict__ r,
-                               double *__restrict__ rec) {
-    __shared__ double red[256];
-    const NetIn n = nets[blockIdx.x];
+// Sums over the squeezing parameters, in two kernels: bound by the FP64 pipe (2
+// lanes per SM and clock), so the transcendental part is spread over blocks of
+// 512 parameters (one block per network left an 8000-mode network on one SM),
+// with sinh from one expm1 (sinh r = (u + u / (u + 1)) / 2, u = e^r - 1) and cosh
+// 2r = 1 + 2 sinh^2 r.  One pass over r, which may lie in host memory: the
+// deviation is summed about the network's first parameter c (r varies about c
+// by the deviation itself, so nothing cancels beyond a few bits).
+// part[net][chunk] = sum r - c, sum (r - c)^2, sum sinh^2, sum sinh^4, min, max.
+constexpr int kFeatChunk = 512;
+constexpr int kFeatPart = 6;
+
+__global__ void __launch_bounds__(256) k_sur_feature_parts(const NetIn *__restrict__ nets,
+                                                           const double *__restrict__ r,
+                                                           int chunks, double *__restrict__ part) {
+    __shared__ double red[8][kFeatPart];
+    const NetIn n = nets[blockIdx.y];
+    const int j0 = blockIdx.x * kFeatChunk;
+    if (j0 >= n.N) return;
     const double *rj = r + n.r0;
-    const double eta = n.t * n.t;
-    double s1 = 0.0, s2 = 0.0, s3 = 0.0, lo = INFINITY, hi = -INFINITY;
-    for (int j = threadIdx.x; j < n.N; j += blockDim.x) {
+    const double c = rj[0];
+    double v[kFeatPart] = {0.0, 0.0, 0.0, 0.0, INFINITY, -INFINITY};
+    auto join = [](double (&a)[kFeatPart], const double (&b)[kFeatPart]) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] += b[q];
+        a[4] = fmin(a[4], b[4]);
+        a[5] = fmax(a[5], b[5]);
+    };
+#pragma unroll
+    for (int t = 0; t < kFeatChunk / 256; ++t) {
+        const int j = j0 + t * 256 + threadIdx.x;
+        if (j >= n.N) break;
         const double x = rj[j];
-        const double sh = sinh(x);
+        const double u = expm1(x);
+        const double sh = 0.5 * (u + (u < 0x1p60 ? u / (u + 1.0) : 1.0));
         const double sh2 = sh * sh;
-        s1 += x;
-        s2 += eta * sh2;
-        s3 += eta * sh2 + eta * eta * sh2 * cosh(2.0 * x);
-        lo = fmin(lo, x);
-        hi = fmax(hi, x);
+        join(v, {x - c, (x - c) * (x - c), sh2, sh2 * sh2, x, x});
     }
-    const double sum_r = block_sum<256>(s1, red);
-    const double mu = block_sum<256>(s2, red);
-    const double var = block_sum<256>(s3, red);
-    // min / max
-    red[threadIdx.x] = lo;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] = fmin(red[threadIdx.x], red[threadIdx.x + w]);
-        __syncthreads();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        double w[kFeatPart];
+#pragma unroll
+        for (int q = 0; q < kFeatPart; ++q) w[q] = __shfl_xor_sync(0xffffffffu, v[q], o);
+        join(v, w);
     }
-    const double rmin = red[0];
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int q = 0; q < kFeatPart; ++q) red[threadIdx.x >> 5][q] = v[q];
     __syncthreads();
-    red[threadIdx.x] = hi;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
-        __syncthreads();
-    }
-    const double rmax = red[0];
-    __syncthreads();
-    const double mean = sum_r / (double)n.N;
-    double d2 = 0.0;
-    for (int j = threadIdx.x; j < n.N; j += blockDim.x) {
-        const double d = rj[j] - mean;
-        d2 += d * d;
-    }
-    const double ss = block_sum<256>(d2, red);
     if (threadIdx.x == 0) {
-        double *o = rec + (size_t)blockIdx.x * kRec;
-        const double s = sqrt(var);
-        o[0] = log((double)n.N);
-        o[1] = log((double)n.M);
-        o[2] = mean;
-        o[3] = sqrt(ss / (double)n.N);
-        o[4] = rmin;
-        o[5] = rmax;
-        o[6] = n.t;
-        o[7] = log2((double)n.K1);
-        o[8] = log(mu);
-        o[9] = log(s);
-        o[10] = mu;
-        o[11] = s;
-        o[12] = (double)n.m_off;
-        o[13] = (double)n.K1;
+        for (int w = 1; w < 8; ++w) join(v, red[w]);
+        double *o = part + ((size_t)blockIdx.y * chunks + blockIdx.x) * kFeatPart;
+#pragma unroll
+        for (int q = 0; q < kFeatPart; ++q) o[q] = v[q];
     }
+}
+
+// One warp per network: its chunks in order, and the record.
+__global__ void k_sur_features(const NetIn *__restrict__ nets, const double *__restrict__ r,
+                               const double *__restrict__ part, int chunks, int count,
+                               double *__restrict__ rec) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (i >= count) return;
+    const NetIn n = nets[i];
+    double v = 0.0;
+    if (lane < kFeatPart) {
+        const double *p = part + (size_t)i * chunks * kFeatPart + lane;
+        v = p[0];
+        for (int c = 1; c * kFeatChunk < n.N; ++c) {
+            const double w = p[c * kFeatPart];
+            v = lane < 4 ? v + w : lane == 4 ? fmin(v, w) : fmax(v, w);
+        }
+    }
+    double t[kFeatPart];
+#pragma unroll
+    for (int q = 0; q < kFeatPart; ++q) t[q] = __shfl_sync(0xffffffffu, v, q);
+    const double eta = n.t * n.t;
+    const double mu = eta * t[2];
+    // sum of eta sinh^2 + eta^2 sinh^2 (1 + 2 sinh^2)
+    const double s = sqrt(mu + eta * mu + 2.0 * eta * eta * t[3]);
+    const double d = t[0] / (double)n.N;
+    double *o = rec + (size_t)i * kRec;
+    // the logarithms side by side in the lanes
+    double x = 1.0;
+    if (lane == 0) x = (double)n.N;
+    if (lane == 1) x = (double)n.M;
+    if (lane == 8) x = mu;
+    if (lane == 9) x = s;
+    const double lg = log(x);
+    if (lane == 0 || lane == 1 || lane == 8 || lane == 9) o[lane] = lg;
+    if (lane == 2) o[2] = r[n.r0] + d;
+    if (lane == 3) o[3] = sqrt(fmax(t[1] / (double)n.N - d * d, 0.0));
+    if (lane == 4) o[4] = t[4];
+    if (lane == 5) o[5] = t[5];
+    if (lane == 6) o[6] = n.t;
+    if (lane == 7) o[7] = (double)(31 - __clz(n.K1));  // a power of two
+    if (lane == 10) o[10] = mu;
+    if (lane == 11) o[11] = s;
+    if (lane == 12) o[12] = (double)n.m_off;
+    if (lane == 13) o[13] = (double)n.K1;
 }
 
 // One block of 32 x kFeat threads: warp f handles feature f.
@@ -196,48 +237,83 @@ __global__ void k_sur_encode(const double *__restrict__ rec, const double *__res
     Y[(size_t)blockIdx.x * 2 * kGrid + threadIdx.x] = (float)(kOutScale * (f - half_phi(x)));
 }
 
-// One block (256 threads) per network: P(m) on the window, then renormalised.
-__global__ void k_sur_decode(const double *__restrict__ rec, const float *__restrict__ Y,
-                             double *__restrict__ P, int64_t ldP) {
-    __shared__ double f[2][kGrid];
+// phi(x_i) / 2 on the output grid (host table, passed by value).
+struct HalfPhi {
+    double v[kGrid];
+};
+
+HalfPhi half_phi_table() {
+    HalfPhi t;
+    for (int i = 0; i < kGrid; ++i) {
+        const double x = kXLo + kDx * (i + 0.5);
+        t.v[i] = 0.5 * kInvSqrt2Pi * std::exp(-0.5 * x * x);
+    }
+    return t;
+}
+
+// P(m) on the window, then renormalised (which also cancels the factor 2 / s of
+// a density): a cluster of kDecodeBlocks blocks (256 threads) per network, the
+// total through distributed shared memory.  Bound by the FP64 pipe: with one
+// block per network and the exponentials, divisions and Hermite basis written
+// out, 4096 counts took 129 us of one SM (under ncu).
+constexpr int kDecodeBlocks = 4;
+
+__global__ void __cluster_dims__(kDecodeBlocks, 1, 1) __launch_bounds__(256)
+    k_sur_decode(const double *__restrict__ rec, const float *__restrict__ Y, const HalfPhi hp,
+                 double *__restrict__ P, int64_t ldP) {
+    __shared__ double f[2][kGrid + 4];  // two zeros before and after the grid
     __shared__ double red[256];
-    const double *q = rec + (size_t)blockIdx.x * kRec;
-    const double mu = q[10], s = q[11];
+    __shared__ double part;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int net = blockIdx.x / kDecodeBlocks, rank = blockIdx.x % kDecodeBlocks;
+    const double *q = rec + (size_t)net * kRec;
+    const double mu = q[10], inv = 1.0 / (q[11] * kDx);
     const int64_t m_off = (int64_t)q[12];
     const int64_t K1 = min((int64_t)q[13], ldP);
-    const float *o = Y + (size_t)blockIdx.x * 2 * kGrid;
-    for (int k = threadIdx.x; k < 2 * kGrid; k += blockDim.x) {
-        const double x = kXLo + kDx * ((k % kGrid) + 0.5);
-        f[k / kGrid][k % kGrid] = (double)o[k] / kOutScale + half_phi(x);
+    const float *o = Y + (size_t)net * 2 * kGrid;
+    for (int k = threadIdx.x; k < 2 * (kGrid + 4); k += 256) {
+        const int p = k / (kGrid + 4), i = k % (kGrid + 4) - 2;
+        f[p][i + 2] = i >= 0 && i < kGrid ? (double)o[p * kGrid + i] / kOutScale + hp.v[i] : 0.0;
     }
     __syncthreads();
-    double *Pn = P + (size_t)blockIdx.x * ldP;
-    double part = 0.0;
-    for (int64_t j = threadIdx.x; j < K1; j += blockDim.x) {
+    double *Pn = P + (size_t)net * ldP;
+    double sum = 0.0;
+    for (int64_t j = rank * 256 + threadIdx.x; j < K1; j += 256 * kDecodeBlocks) {
         const int64_t m = m_off + j;
-        const int p = (int)(m & 1);
-        const double g = ((m - mu) / s - (kXLo + 0.5 * kDx)) / kDx;
+        const double g = (m - mu) * inv - (kXLo + 0.5 * kDx) / kDx;
         double v = 0.0;
         if (g >= 0.0 && g <= kGrid - 1) {
             const double g0 = floor(g);
-            const int i0 = (int)g0;
             const double u = g - g0;
-            double y[4];
-#pragma unroll
-            for (int d = 0; d < 4; ++d) {
-                const int ii = i0 + d - 1;
-                y[d] = (ii >= 0 && ii < kGrid) ? f[p][ii] : 0.0;
-            }
-            v = 2.0 / s * fmax(cr(y[0], y[1], y[2], y[3], u), 0.0);
+            // Catmull-Rom (cr) in powers of u
+            const double *y = &f[m & 1][(int)g0 + 1];
+            const double c1 = 0.5 * (y[2] - y[0]);
+            const double d = y[1] - y[2];
+            const double c3 = 0.5 * (y[3] - y[0]) + 1.5 * d;
+            const double c2 = -(c1 + c3) - d;
+            v = fmax(fma(fma(fma(c3, u, c2), u, c1), u, y[1]), 0.0);
         }
         Pn[j] = v;
-        part += v;
+        sum += v;
     }
-    const double total = block_sum<256>(part, red);
+    sum = block_sum<256>(sum, red);
+    if (threadIdx.x == 0) part = sum;
+    cluster.sync();
+    double total = 0.0;
+#pragma unroll
+    for (int b = 0; b < kDecodeBlocks; ++b) total += *cluster.map_shared_rank(&part, b);
+    cluster.sync();  // every block has read the parts
     if (total > 0.0) {
-        const double inv = 1.0 / total;
-        for (int64_t j = threadIdx.x; j < K1; j += blockDim.x) Pn[j] *= inv;
+        const double scale = 1.0 / total;
+        for (int64_t j = rank * 256 + threadIdx.x; j < K1; j += 256 * kDecodeBlocks) Pn[j] *= scale;
     }
+}
+
+// Whether every r[j] is finite and positive (written to vectorise).
+__attribute__((optimize("O3"))) bool all_positive(const double *r, int64_t n) {
+    int64_t bad = 0;
+    for (int64_t j = 0; j < n; ++j) bad += !(r[j] > 0.0 && r[j] <= 1.7976931348623157e308);
+    return bad == 0;
 }
 
 int check_records(int count, const void *feat) {
@@ -273,32 +349,55 @@ int gbs_surrogate_features(int count, const int *N, const int *M, const double *
         h[(size_t)i] = NetIn{t[i], m_off[i], r_off[i], N[i], M[i], K1[i], 0};
     }
     const int64_t nr = r_off[count];
-    for (int64_t j = 0; j < nr; ++j)
-        if (!(std::isfinite(r[j]) && r[j] > 0.0))
-            return set_error(GBS_EINVAL, "r[%lld] must be finite and > 0", (long long)j);
+    if (!all_positive(r, nr))
+        for (int64_t j = 0; j < nr; ++j)
+            if (!(std::isfinite(r[j]) && r[j] > 0.0))
+                return set_error(GBS_EINVAL, "r[%lld] must be finite and > 0", (long long)j);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    NetIn *d_nets = nullptr;
-    double *d_r = nullptr;
-    if (cudaMalloc(&d_nets, sizeof(NetIn) * (size_t)count) != cudaSuccess ||
-        cudaMalloc(&d_r, sizeof(double) * (size_t)nr) != cudaSuccess) {
+    int Nmax = 0;
+    for (int i = 0; i < count; ++i) Nmax = N[i] > Nmax ? N[i] : Nmax;
+    const int chunks = (Nmax + kFeatChunk - 1) / kFeatChunk;
+    // Where the device addresses pageable host memory (Grace), r is read in
+    // place, once, over the host link; else it is uploaded.  The call
+    // synchronises before it returns, so r is not read afterwards.
+    int dev = 0, direct = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&direct, cudaDevAttrPageableMemoryAccess, dev) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(d_nets);
-        return set_error(GBS_ENOMEM, "upload buffers for the features");
+        direct = 0;
     }
-    rc = GBS_OK;
+    // stream-ordered work space: no allocation by the driver on each call
+    void *d_nets = nullptr, *d_r = nullptr, *d_part = nullptr;
+    if ((rc = pool_alloc(&d_nets, sizeof(NetIn) * (size_t)count, s, "network parameters")) ||
+        (!direct && (rc = pool_alloc(&d_r, sizeof(double) * (size_t)nr, s, "squeezing parameters"))) ||
+        (rc = pool_alloc(&d_part, sizeof(double) * (size_t)count * chunks * kFeatPart, s,
+                         "feature sums"))) {
+        pool_free_raw(d_nets, s);
+        pool_free_raw(d_r, s);
+        return rc;
+    }
     if (cudaMemcpyAsync(d_nets, h.data(), sizeof(NetIn) * (size_t)count, cudaMemcpyHostToDevice, s) !=
             cudaSuccess ||
-        cudaMemcpyAsync(d_r, r, sizeof(double) * (size_t)nr, cudaMemcpyHostToDevice, s) != cudaSuccess)
+        (!direct && cudaMemcpyAsync(d_r, r, sizeof(double) * (size_t)nr, cudaMemcpyHostToDevice, s) !=
+                        cudaSuccess))
         rc = set_error(GBS_ECUDA, "upload of the network parameters failed");
     if (!rc) {
-        k_sur_features<<<count, 256, 0, s>>>(d_nets, d_r, feat_dev);
+        const double *rp = direct ? r : static_cast<const double *>(d_r);
+        const NetIn *np = static_cast<const NetIn *>(d_nets);
+        double *pp = static_cast<double *>(d_part);
+        // grid.y holds at most 65535 networks
+        for (int i0 = 0; i0 < count; i0 += 65535)
+            k_sur_feature_parts<<<dim3((unsigned)chunks, (unsigned)std::min(65535, count - i0)), 256, 0,
+                                  s>>>(np + i0, rp, chunks, pp + (size_t)i0 * chunks * kFeatPart);
+        k_sur_features<<<(count + 7) / 8, 256, 0, s>>>(np, rp, pp, chunks, count, feat_dev);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = set_error(GBS_ECUDA, "feature kernel: %s", cudaGetErrorString(e));
     }
     if (cudaStreamSynchronize(s) != cudaSuccess && !rc)
         rc = set_error(GBS_ECUDA, "feature kernel failed");
-    cudaFree(d_nets);
-    cudaFree(d_r);
+    pool_free_raw(d_nets, s);
+    pool_free_raw(d_r, s);
+    pool_free_raw(d_part, s);
     return rc;
 }
 
@@ -338,7 +437,9 @@ int gbs_surrogate_decode(int count, const double *feat_dev, const float *Y_dev, 
     int rc;
     if ((rc = check_records(count, feat_dev))) return rc;
     if (!P_dev || !Y_dev || ldP < 1) return set_error(GBS_EINVAL, "NULL device array or ldP < 1");
-    k_sur_decode<<<count, 256, 0, static_cast<cudaStream_t>(stream)>>>(feat_dev, Y_dev, P_dev, ldP);
+    static const HalfPhi hp = half_phi_table();
+    k_sur_decode<<<count * kDecodeBlocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        feat_dev, Y_dev, hp, P_dev, ldP);
     GBS_LAUNCH_CHECK();
     return GBS_OK;
 }
