@@ -205,6 +205,7 @@ void release_all(gbs_net *net) {
     net_free(net, net->d_sq64);
     net_free(net, net->d_sq32);
     net_free(net, net->d_T64);
+    net_free(net, net->d_T32);
     net_free(net, net->d_Aq);
     net_free(net, net->d_rowexp);
     net_free(net, net->d_colexp);
@@ -674,6 +675,12 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
         rc = finish_device_T(net, d_bad);
         net_free(net, d_bad);
         if (rc) return fail(rc);
+        if (precision == GBS_FP32) {
+            if ((rc = net_alloc(net, &net->d_T32, fp32_A_floats(N, net->mtiles), "T32")) ||
+                (rc = launch_t32_tiles(net)))
+                return fail(rc);
+            net_free(net, net->d_T64);
+        }
         if (precision == GBS_FP64 && N >= kF64tcMinN && (rc = make_f64tc_operand(net, sq64)))
             return fail(rc);
     } else {
@@ -706,7 +713,8 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
     // chunk workspace
     net->chunk = pick_chunk(net);
     if (simt_precision(precision)) {
-        net->B_bytes = net->d_Aq ? f64tc_B_bytes(N, net->chunk)
+        net->B_bytes = net->d_Aq    ? f64tc_B_bytes(N, net->chunk)
+                       : net->d_T32 ? fp32_B_bytes(N, net->chunk)
                                  : (size_t)net->chunk * 2 * N * sizeof(double);
     } else {
         const int64_t tiles = (net->chunk + kTcTileSamples - 1) / kTcTileSamples;

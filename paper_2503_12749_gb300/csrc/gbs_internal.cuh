@@ -45,6 +45,8 @@ constexpr double kSkipLog = 41.58883083359672;    // 60 * ln 2
 constexpr double kSkipLogDf = 32.57791748631743;  // 47 * ln 2
 constexpr int kFp64TileModes = 64;              // output modes per FP64 GEMM tile
 constexpr int kFp64TileSamples = 32;            // samples per FP64 GEMM tile
+constexpr int kFp32TileSamples = 64;            // samples per FP32 GEMM tile
+constexpr int kFp32BlockK = 16;                 // input modes per FP32 GEMM stage
 // Input modes from which the FP64 GEMM runs as digit products on the tensor
 // cores (k_gemm_f64tc.cu): one whole K step.  It is the faster one at every
 // size (N = M = 16, 16384 trajectories: 0.054 against 0.150 ms), but its
@@ -140,9 +142,9 @@ struct Profiler {
     int64_t launches[GBS_NPHASES] = {};
 };
 
-// The SIMT precisions (GBS_FP64, GBS_FP32) share the FP64 sampler, network
-// operand, generating functions and inversion; only the GEMM's arithmetic
-// differs.  The BF16 split precisions run the tcgen05 path.
+// GBS_FP64 and GBS_FP32 share the FP64 sampler's
+// arithmetic, generating functions and inversion; only the GEMM's arithmetic
+// (and the precision its operands are stored in) differs.  The BF16 split precisions run the tcgen05 path.
 inline bool simt_precision(int precision) {
     return precision == GBS_FP64 || precision == GBS_FP32;
 }
@@ -160,6 +162,10 @@ struct gbs_net {
 
     // FP64 network operand: [M][2][N], row (i,0) = Re T_i., (i,1) = Im T_i.
     double *d_T64 = nullptr;
+
+    // GBS_FP32: the network operand as FP32 tiles (k_gemm_fp32.cu); d_B then
+    // holds FP32 tiles too and d_T64 is not kept
+    float *d_T32 = nullptr;
 
     // GBS_FP64 on the tensor cores (k_gemm_f64tc.cu): the network operand as
     // digit tiles, its row exponents (mtiles * 128), the input modes'
@@ -264,6 +270,11 @@ SampleJob sample_job_bf16(gbs_net *net, void *B, double *n, uint64_t seed, uint6
 
 // Propagation GEMM with the fused occupation epilogue -> nS_part[mtiles][chunk].
 int launch_gemm_fp64(gbs_net *net, int64_t count, OccOut64 occ = OccOut64());
+// The FP32 GEMM: tiles of T from d_T64, sizes of the two operands.
+int launch_t32_tiles(gbs_net *net);
+int launch_gemm_fp32(gbs_net *net, int64_t count, OccOut64 occ);
+size_t fp32_A_floats(int N, int mtiles);
+size_t fp32_B_bytes(int N, int64_t chunk);
 // The FP64 GEMM on the tensor cores.  Exponents of the input modes from the
 // sampler coefficients (false: outside the range the digits are used for);
 // digit tiles of T from d_T64 (*d_bad counts rows outside the range); bytes

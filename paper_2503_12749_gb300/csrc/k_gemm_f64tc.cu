@@ -72,15 +72,6 @@ constexpr uint64_t kWaitNs = 2000000000ull;
 // make one wave of 152 CTAs, the most square split of its operand traffic
 constexpr int kBand = 8;
 
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes,
-                                          uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            dst),
-        "l"(src), "r"(bytes), "r"(bar)
-        : "memory");
-}
-
 // K-major operand without swizzle: core matrices of 8 rows x 16 bytes; the
 // two of a 16-wide K step 128 bytes apart (leading offset), 8-row groups 256
 // bytes apart (stride offset); descriptor version 1 (bit 46).
@@ -201,8 +192,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint32_t fb = ptx::smem_u32(&full[stage]);
                     uint8_t *s = smem + stage * kStageBytes;
                     ptx::mbar_arrive_expect_tx(fb, kStageBytes);
-                    bulk_load(ptx::smem_u32(s), a + (size_t)kb * kAStage, kAStage, fb);
-                    bulk_load(ptx::smem_u32(s + kAStage), b + (size_t)kb * kBStage, kBStage, fb);
+                    ptx::bulk_load(ptx::smem_u32(s), a + (size_t)kb * kAStage, kAStage, fb);
+                    ptx::bulk_load(ptx::smem_u32(s + kAStage), b + (size_t)kb * kBStage, kBStage, fb);
                     used |= 1u << stage;
                     last = (last & ~(1u << stage)) | (phase << stage);
                     if (++stage == kStages) {

@@ -12,7 +12,8 @@
 // matrix-P and +P estimators (both use the +P sampling procedure).
 //
 // Layouts written:
-//   FP64 path: B[e][c][N] doubles, c = 0 (alpha), 1 (beta).
+//   FP64 path: digit tiles (f64tc.cuh), or, for the networks the tensor cores do
+//   not take, B[e][c][N] doubles, c = 0 (alpha), 1 (beta); FP32 path: FP32 tiles.
 //   BF16 path: per 128-trajectory tile, 256 rows (128 alpha rows, then 128
 //   beta rows); planes B0 = bf16(x), B1 = bf16(x - B0), B2 = bf16(x - B0 -
 //   B1) stored plane-major, each plane K-blocked [ldK / 32][rows][32]
@@ -73,6 +74,45 @@ __global__ void k_sample_fp64(const double2 *__restrict__ sq, int N, uint64_t se
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
         if (lane == 0) n_out[i] = part;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// FP32 path: the FP64 samples rounded to FP32 tiles [64 trajectories][K block]
+// [16 k][64 alpha, 64 beta] (k_gemm_fp32.cu).  A block holds 32 trajectories, a
+// lane each, and its 8 warps take every eighth mode (128-byte stores).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_sample_fp32(const double2 *__restrict__ sq, int N, int KB,
+                                                     uint64_t seed, uint64_t e0, int64_t count,
+                                                     float *__restrict__ B,
+                                                     double *__restrict__ n_out) {
+    __shared__ double s_n[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    const uint64_t e = e0 + (uint64_t)i;
+    constexpr int kRow = 2 * kFp32TileSamples;
+    float *tile = B + (size_t)(i / kFp32TileSamples) * KB * kFp32BlockK * kRow + i % kFp32TileSamples;
+    double part = 0.0;
+    if (i < count)
+        for (int j = warp; j < KB * kFp32BlockK; j += 8) {
+            double a = 0.0, b = 0.0;
+            if (j < N) {
+                double w1, w2;
+                normals_fp64(seed, e, (uint32_t)j, w1, w2);
+                const double2 q = sq[j];
+                a = q.x * w1 + q.y * w2;
+                b = q.x * w1 - q.y * w2;
+                part += a * b;
+            }
+            tile[(size_t)j * kRow] = (float)a;
+            tile[(size_t)j * kRow + kFp32TileSamples] = (float)b;
+        }
+    s_n[warp][lane] = part;
+    __syncthreads();
+    if (warp == 0 && i < count) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) part += s_n[w][lane];
+        n_out[i] = part;
     }
 }
 
@@ -171,6 +211,13 @@ int launch_sample_fp64(gbs_net *net, uint64_t seed, uint64_t e0, int64_t count) 
         k_sample_f64tc<<<(unsigned)((count + 7) / 8), 128, 0, net->stream>>>(
             net->d_sq64, net->d_colexp, net->N, f64tc_kblocks(net->N), seed, e0, count,
             static_cast<uint8_t *>(net->d_B), net->d_n);
+        GBS_LAUNCH_CHECK();
+        return GBS_OK;
+    }
+    if (net->d_T32) {
+        k_sample_fp32<<<(unsigned)((count + 31) / 32), 256, 0, net->stream>>>(
+            net->d_sq64, net->N, (net->N + kFp32BlockK - 1) / kFp32BlockK, seed, e0, count,
+            static_cast<float *>(net->d_B), net->d_n);
         GBS_LAUNCH_CHECK();
         return GBS_OK;
     }
