@@ -204,6 +204,7 @@ void release_all(gbs_net *net) {
     if (net->tc) tc_plan_destroy(net);
     net_free(net, net->d_sq64);
     net_free(net, net->d_sq32);
+    net_free(net, net->d_ntab);
     net_free(net, net->d_T64);
     net_free(net, net->d_T32);
     net_free(net, net->d_Aq);
@@ -675,6 +676,10 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
         rc = finish_device_T(net, d_bad);
         net_free(net, d_bad);
         if (rc) return fail(rc);
+        if ((rc = pool_alloc(reinterpret_cast<void **>(&net->d_ntab), norm_tab_bytes(), net->stream,
+                             "normal tables")) ||
+            (rc = upload_norm_tab(net)))
+            return fail(rc);
         if (precision == GBS_FP32) {
             if ((rc = net_alloc(net, &net->d_T32, fp32_A_floats(N, net->mtiles), "T32")) ||
                 (rc = launch_t32_tiles(net)))

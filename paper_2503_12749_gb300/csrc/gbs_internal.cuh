@@ -78,6 +78,7 @@ struct WindowD {
 // ---------------------------------------------------------------------------
 // The network object behind gbs_net_t
 // ---------------------------------------------------------------------------
+struct NormTab;  // tables of the FP64 normals (normal_f64.cuh)
 struct TcPlan;  // tcgen05 GEMM plan (tensor maps, tiling), defined in k_gemm_tc.cu
 
 // Operand description of one network for the (grouped) tcgen05 GEMM, kept in
@@ -159,6 +160,9 @@ struct gbs_net {
     // per-mode sampler coefficients: (sqrt(s+/2), sqrt(s-/2)), s+- = sinh r e^{+-r}
     double2 *d_sq64 = nullptr;
     float2 *d_sq32 = nullptr;
+
+    // tables of the FP64 sampler's normals (GBS_FP64, GBS_FP32)
+    gbs::NormTab *d_ntab = nullptr;
 
     // FP64 network operand: [M][2][N], row (i,0) = Re T_i., (i,1) = Im T_i.
     double *d_T64 = nullptr;
@@ -264,6 +268,9 @@ void pool_free_raw(void *p, cudaStream_t stream);
 // Sampler: writes the sample operand for trajectories e0..e0+count-1 and n[].
 int launch_sample_fp64(gbs_net *net, uint64_t seed, uint64_t e0, int64_t count);
 int launch_sample_bf16(gbs_net *net, uint64_t seed, uint64_t e0, int64_t count);
+// The FP64 normals' tables into net->d_ntab.
+int upload_norm_tab(gbs_net *net);
+size_t norm_tab_bytes();
 // The BF16 sampler's job for trajectories e0..e0+count-1 into (B, n).
 SampleJob sample_job_bf16(gbs_net *net, void *B, double *n, uint64_t seed, uint64_t e0,
                           int64_t count);

@@ -23,36 +23,43 @@
 // 3-product GEMM, which sample the next chunk.
 #include "gbs_internal.cuh"
 #include "f64tc.cuh"
+#include "normal_f64.cuh"
 #include "sampler_dev.cuh"
+
+#include <algorithm>
 
 namespace gbs {
 namespace {
 
-// 53-bit uniform in (0,1): 27 high bits of a, 26 high bits of b, +1/2 unit.
-__device__ __forceinline__ double uniform53(uint32_t a, uint32_t b) {
-    const double hi = (double)(a >> 5);
-    const double lo = (double)(b >> 6);
-    return (hi * 67108864.0 + lo + 0.5) * (1.0 / 9007199254740992.0);
-}
-
-__device__ __forceinline__ void normals_fp64(uint64_t seed, uint64_t e, uint32_t j, double &w1,
-                                             double &w2) {
+// Both amplitudes of (trajectory e, input mode j).
+__device__ __forceinline__ void amplitudes(const NormTab &T, uint64_t seed, uint64_t e, uint32_t j,
+                                           double2 q, double &a, double &b) {
     uint32_t c0 = (uint32_t)e, c1 = (uint32_t)(e >> 32), c2 = j, c3 = 0u;
     samp::philox4x32_10(c0, c1, c2, c3, (uint32_t)seed, (uint32_t)(seed >> 32));
-    const double u1 = uniform53(c0, c1);
-    const double u2 = uniform53(c2, c3);
-    const double rho = sqrt(-2.0 * log(u1));
-    double s, c;
-    sincospi(2.0 * u2, &s, &c);
-    w1 = rho * c;
-    w2 = rho * s;
+    double w1, w2;
+    nrm::normals(c0, c1, c2, c3, T, w1, w2);
+    const double t = q.y * w2;
+    a = fma(q.x, w1, t);
+    b = fma(q.x, w1, -t);
+}
+
+// The tables in shared memory (lanes read them at unrelated indexes).
+__device__ __forceinline__ void load_tab(NormTab &sh, const NormTab *__restrict__ tab) {
+    static_assert(sizeof(NormTab) % 16 == 0, "table copied in 16-byte words");
+    const uint4 *src = reinterpret_cast<const uint4 *>(tab);
+    uint4 *dst = reinterpret_cast<uint4 *>(&sh);
+    for (int t = threadIdx.x; t < (int)(sizeof(NormTab) / 16); t += blockDim.x) dst[t] = src[t];
+    __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
 // FP64 path: one warp per trajectory, lanes stride over input modes.
 // ---------------------------------------------------------------------------
-__global__ void k_sample_fp64(const double2 *__restrict__ sq, int N, uint64_t seed, uint64_t e0,
-                              int64_t count, double *__restrict__ B, double *__restrict__ n_out) {
+__global__ void k_sample_fp64(const double2 *__restrict__ sq, const NormTab *__restrict__ tab, int N,
+                              uint64_t seed, uint64_t e0, int64_t count, double *__restrict__ B,
+                              double *__restrict__ n_out) {
+    __shared__ __align__(16) NormTab sh;
+    load_tab(sh, tab);
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -62,11 +69,8 @@ __global__ void k_sample_fp64(const double2 *__restrict__ sq, int N, uint64_t se
         double *row_b = row_a + N;
         double part = 0.0;
         for (int j = lane; j < N; j += 32) {
-            double w1, w2;
-            normals_fp64(seed, e, (uint32_t)j, w1, w2);
-            const double2 q = sq[j];
-            const double a = q.x * w1 + q.y * w2;
-            const double b = q.x * w1 - q.y * w2;
+            double a, b;
+            amplitudes(sh, seed, e, (uint32_t)j, sq[j], a, b);
             row_a[j] = a;
             row_b[j] = b;
             part += a * b;
@@ -82,104 +86,109 @@ __global__ void k_sample_fp64(const double2 *__restrict__ sq, int N, uint64_t se
 // [16 k][64 alpha, 64 beta] (k_gemm_fp32.cu).  A block holds 32 trajectories, a
 // lane each, and its 8 warps take every eighth mode (128-byte stores).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_sample_fp32(const double2 *__restrict__ sq, int N, int KB,
-                                                     uint64_t seed, uint64_t e0, int64_t count,
-                                                     float *__restrict__ B,
-                                                     double *__restrict__ n_out) {
+__global__ void __launch_bounds__(256)
+    k_sample_fp32(const double2 *__restrict__ sq, const NormTab *__restrict__ tab, int N, int KB,
+                  uint64_t seed, uint64_t e0, int64_t count, float *__restrict__ B,
+                  double *__restrict__ n_out) {
+    __shared__ __align__(16) NormTab sh;
     __shared__ double s_n[8][32];
+    load_tab(sh, tab);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
-    const uint64_t e = e0 + (uint64_t)i;
     constexpr int kRow = 2 * kFp32TileSamples;
-    float *tile = B + (size_t)(i / kFp32TileSamples) * KB * kFp32BlockK * kRow + i % kFp32TileSamples;
-    double part = 0.0;
-    if (i < count)
-        for (int j = warp; j < KB * kFp32BlockK; j += 8) {
-            double a = 0.0, b = 0.0;
-            if (j < N) {
-                double w1, w2;
-                normals_fp64(seed, e, (uint32_t)j, w1, w2);
-                const double2 q = sq[j];
-                a = q.x * w1 + q.y * w2;
-                b = q.x * w1 - q.y * w2;
-                part += a * b;
+    for (int64_t i0 = (int64_t)blockIdx.x * 32; i0 < count; i0 += (int64_t)gridDim.x * 32) {
+        const int64_t i = i0 + lane;
+        float *tile =
+            B + (size_t)(i / kFp32TileSamples) * KB * kFp32BlockK * kRow + i % kFp32TileSamples;
+        double part = 0.0;
+        if (i < count)
+            for (int j = warp; j < KB * kFp32BlockK; j += 8) {
+                double a = 0.0, b = 0.0;
+                if (j < N) {
+                    amplitudes(sh, seed, e0 + (uint64_t)i, (uint32_t)j, sq[j], a, b);
+                    part = fma(a, b, part);
+                }
+                tile[(size_t)j * kRow] = (float)a;
+                tile[(size_t)j * kRow + kFp32TileSamples] = (float)b;
             }
-            tile[(size_t)j * kRow] = (float)a;
-            tile[(size_t)j * kRow + kFp32TileSamples] = (float)b;
-        }
-    s_n[warp][lane] = part;
-    __syncthreads();
-    if (warp == 0 && i < count) {
+        s_n[warp][lane] = part;
+        __syncthreads();
+        if (warp == 0 && i < count) {
 #pragma unroll
-        for (int w = 1; w < 8; ++w) part += s_n[w][lane];
-        n_out[i] = part;
+            for (int w = 1; w < 8; ++w) part += s_n[w][lane];
+            n_out[i] = part;
+        }
+        __syncthreads();
     }
 }
 
 // ---------------------------------------------------------------------------
-// FP64 path on the tensor cores: the digit tiles of f64tc.cuh.  A block holds
-// 8 trajectories (one core matrix) and its 4 warps take 16 groups of 8
-// consecutive modes per pass, a lane one group of one trajectory: it stores 16
-// bytes per digit, the 8 lanes of a group one 128-byte core matrix.
+// FP64 path on the tensor cores: the digit tiles of f64tc.cuh.  `wpg` of a
+// block's 8 warps (1, 2, 4 or 8, by the number of modes) hold 8 trajectories (one
+// core matrix); a warp takes 4 groups of 8 consecutive modes per pass, a lane one
+// group of one trajectory: it stores 16 bytes per digit, the 8 lanes of a group
+// one 128-byte core matrix.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_sample_f64tc(const double2 *__restrict__ sq,
-                                                      const int *__restrict__ col_exp, int N,
-                                                      int KB, uint64_t seed, uint64_t e0,
-                                                      int64_t count, uint8_t *__restrict__ B,
-                                                      double *__restrict__ n_out) {
+__global__ void __launch_bounds__(256, 2)
+    k_sample_f64tc(const double2 *__restrict__ sq, const NormTab *__restrict__ tab,
+                   const int *__restrict__ col_exp, int N, int KB, int wpg, uint64_t seed,
+                   uint64_t e0, int64_t count, uint8_t *__restrict__ B, double *__restrict__ n_out) {
     using namespace f64tc;
-    __shared__ double s_n[4][8];
+    __shared__ __align__(16) NormTab sh;
+    __shared__ double s_n[8][8];
+    load_tab(sh, tab);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 8 + (lane & 7);
-    const uint64_t e = e0 + (uint64_t)i;
-    const int row = (int)(i & 15);
-    uint8_t *tile = B + (size_t)(i / kTrajTile) * KB * kBStage + ((i >> 4) & 1) * kBSub;
-    double part = 0.0;
-    if (i < count)
-        for (int oct = warp * 4 + (lane >> 3); oct < 2 * KB; oct += 16) {
-            uint32_t da[kDigits][4], db[kDigits][4];
+    const int per = 8 / wpg * 8;  // trajectories per block and turn
+    for (int64_t i0 = (int64_t)blockIdx.x * per; i0 < count; i0 += (int64_t)gridDim.x * per) {
+        const int64_t i = i0 + warp / wpg * 8 + (lane & 7);
+        const uint64_t e = e0 + (uint64_t)i;
+        const int row = (int)(i & 15);
+        uint8_t *tile = B + (size_t)(i / kTrajTile) * KB * kBStage + ((i >> 4) & 1) * kBSub;
+        double part = 0.0;
+        if (i < count)
+            for (int oct = (warp & (wpg - 1)) * 4 + (lane >> 3); oct < 2 * KB; oct += 4 * wpg) {
+                uint32_t da[kDigits][4], db[kDigits][4];
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const int j = oct * 8 + t;
-                uint16_t pa[kDigits] = {}, pb[kDigits] = {};
-                if (j < N) {
-                    double w1, w2;
-                    normals_fp64(seed, e, (uint32_t)j, w1, w2);
-                    const double2 q = sq[j];
-                    const double a = q.x * w1 + q.y * w2;
-                    const double b = q.x * w1 - q.y * w2;
-                    const int s = 55 - col_exp[j];
-                    digits_bf16(to_fixed(a, s), pa);
-                    digits_bf16(to_fixed(b, s), pb);
-                    part += a * b;
-                }
+                for (int q = 0; q < kDigits; ++q)
 #pragma unroll
-                for (int q = 0; q < kDigits; ++q) {
-                    if (t & 1) {
-                        da[q][t >> 1] |= (uint32_t)pa[q] << 16;
-                        db[q][t >> 1] |= (uint32_t)pb[q] << 16;
-                    } else {
-                        da[q][t >> 1] = pa[q];
-                        db[q][t >> 1] = pb[q];
+                    for (int t = 0; t < 4; ++t) da[q][t] = db[q][t] = 0u;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    const int j = oct * 8 + t;
+                    if (j < N) {
+                        double a, b;
+                        amplitudes(sh, seed, e, (uint32_t)j, sq[j], a, b);
+                        part = fma(a, b, part);
+                        const int s = 55 - col_exp[j];
+                        uint16_t pa[kDigits], pb[kDigits];
+                        digits_bf16(to_fixed(a, s), pa);
+                        digits_bf16(to_fixed(b, s), pb);
+#pragma unroll
+                        for (int q = 0; q < kDigits; ++q) {
+                            da[q][t >> 1] |= (uint32_t)pa[q] << (16 * (t & 1));
+                            db[q][t >> 1] |= (uint32_t)pb[q] << (16 * (t & 1));
+                        }
                     }
                 }
-            }
-            uint8_t *p = tile + (size_t)(oct >> 1) * kBStage;
-            const int k = (oct & 1) * 8;
+                uint8_t *p = tile + (size_t)(oct >> 1) * kBStage;
+                const int k = (oct & 1) * 8;
 #pragma unroll
-            for (int q = 0; q < kDigits; ++q) {
-                *reinterpret_cast<uint4 *>(p + q * kBSlice + core_offset(row, k)) =
-                    make_uint4(da[q][0], da[q][1], da[q][2], da[q][3]);
-                *reinterpret_cast<uint4 *>(p + q * kBSlice + core_offset(16 + row, k)) =
-                    make_uint4(db[q][0], db[q][1], db[q][2], db[q][3]);
+                for (int q = 0; q < kDigits; ++q) {
+                    *reinterpret_cast<uint4 *>(p + q * kBSlice + core_offset(row, k)) =
+                        make_uint4(da[q][0], da[q][1], da[q][2], da[q][3]);
+                    *reinterpret_cast<uint4 *>(p + q * kBSlice + core_offset(16 + row, k)) =
+                        make_uint4(db[q][0], db[q][1], db[q][2], db[q][3]);
+                }
             }
+        part += __shfl_xor_sync(0xffffffffu, part, 8);
+        part += __shfl_xor_sync(0xffffffffu, part, 16);
+        if (lane < 8) s_n[warp][lane] = part;
+        __syncthreads();
+        if ((warp & (wpg - 1)) == 0 && lane < 8 && i < count) {
+            for (int w = 1; w < wpg; ++w) part += s_n[warp + w][lane];
+            n_out[i] = part;
         }
-    part += __shfl_xor_sync(0xffffffffu, part, 8);
-    part += __shfl_xor_sync(0xffffffffu, part, 16);
-    if (lane < 8) s_n[warp][lane] = part;
-    __syncthreads();
-    if (threadIdx.x < 8 && i < count)
-        n_out[i] = (s_n[0][lane] + s_n[1][lane]) + (s_n[2][lane] + s_n[3][lane]);
+        __syncthreads();
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -208,25 +217,39 @@ int launch_sample_fp64(gbs_net *net, uint64_t seed, uint64_t e0, int64_t count) 
     net->pre_valid = false;  // the operands are overwritten
     if (count <= 0) return GBS_OK;
     if (net->d_Aq) {
-        k_sample_f64tc<<<(unsigned)((count + 7) / 8), 128, 0, net->stream>>>(
-            net->d_sq64, net->d_colexp, net->N, f64tc_kblocks(net->N), seed, e0, count,
-            static_cast<uint8_t *>(net->d_B), net->d_n);
-        GBS_LAUNCH_CHECK();
-        return GBS_OK;
+        // modes in groups of 8, 4 groups per warp and pass
+        const int KB = f64tc_kblocks(net->N);
+        int wpg = 1;
+        while (wpg < 8 && wpg * 4 < 2 * KB) wpg *= 2;
+        const int64_t blocks = (count + 64 / wpg - 1) / (64 / wpg);
+        k_sample_f64tc<<<(unsigned)std::min<int64_t>(blocks, 2 * (int64_t)net->sm_count), 256, 0,
+                         net->stream>>>(net->d_sq64, net->d_ntab, net->d_colexp, net->N, KB, wpg,
+                                        seed, e0, count, static_cast<uint8_t *>(net->d_B), net->d_n);
+    } else if (net->d_T32) {
+        k_sample_fp32<<<(unsigned)std::min<int64_t>((count + 31) / 32, 8 * (int64_t)net->sm_count), 256,
+                        0, net->stream>>>(net->d_sq64, net->d_ntab, net->N,
+                                          (net->N + kFp32BlockK - 1) / kFp32BlockK, seed, e0, count,
+                                          static_cast<float *>(net->d_B), net->d_n);
+    } else {
+        k_sample_fp64<<<grid_for_warps(net, count, 256), 256, 0, net->stream>>>(
+            net->d_sq64, net->d_ntab, net->N, seed, e0, count, static_cast<double *>(net->d_B),
+            net->d_n);
     }
-    if (net->d_T32) {
-        k_sample_fp32<<<(unsigned)((count + 31) / 32), 256, 0, net->stream>>>(
-            net->d_sq64, net->N, (net->N + kFp32BlockK - 1) / kFp32BlockK, seed, e0, count,
-            static_cast<float *>(net->d_B), net->d_n);
-        GBS_LAUNCH_CHECK();
-        return GBS_OK;
-    }
-    const int threads = 256;
-    k_sample_fp64<<<grid_for_warps(net, count, threads), threads, 0, net->stream>>>(
-        net->d_sq64, net->N, seed, e0, count, static_cast<double *>(net->d_B), net->d_n);
     GBS_LAUNCH_CHECK();
     return GBS_OK;
 }
+
+int upload_norm_tab(gbs_net *net) {
+    static const NormTab T = [] {
+        NormTab t;
+        fill_norm_tab(t);
+        return t;
+    }();
+    GBS_CUDA_TRY(cudaMemcpyAsync(net->d_ntab, &T, sizeof(T), cudaMemcpyHostToDevice, net->stream));
+    return GBS_OK;
+}
+
+size_t norm_tab_bytes() { return sizeof(NormTab); }
 
 SampleJob sample_job_bf16(gbs_net *net, void *B, double *n, uint64_t seed, uint64_t e0,
                           int64_t count) {
