@@ -119,17 +119,17 @@ __device__ __forceinline__ Tile tile_of(int t, int mtiles, int stiles) {
     return r;
 }
 
-// Sum over the 32 lanes of 32 values per lane: lane l returns the sum of
-// value l, in a fixed order.
-__device__ __forceinline__ double transpose_sum(double (&v)[32], int lane) {
+// Sum over the 16 lanes of the same parity of 16 values per lane: lanes 2 q and
+// 2 q + 1 return their parity's sum of value q, in a fixed order.
+__device__ __forceinline__ double transpose_sum(double (&v)[16], int lane) {
 #pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        const bool up = (lane & w) != 0;
+    for (int w = 8; w >= 1; w >>= 1) {
+        const bool up = (lane & (2 * w)) != 0;
 #pragma unroll
         for (int i = 0; i < w; ++i) {
             const double send = up ? v[i] : v[i + w];
             const double keep = up ? v[i + w] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * w);
         }
     }
     return v[0];
@@ -245,22 +245,27 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 desc_k_plain(ptx::smem_u32(s + kAStage + sub * kBSub));
                             const uint32_t d = tmem + (uint32_t)sub * 256u;
                             const uint32_t acc = (first && q == 0) ? 0u : 1u;
-                            // digit p of A against digits 0..min(6, 7 - p) of B
-                            ptx::mma_bf16(d, da, db, ptx::idesc_bf16_f32(128, 224), acc);
+                            // digit p of A against digits 0..min(6, 7 - p) of B; the
+                            // long products last, so that the pipe has work while
+                            // the next stage's barrier is polled
                             if (acc) {
-                                ptx::mma_bf16(d + 32u, da + (kASlice >> 4), db,
-                                              ptx::idesc_bf16_f32(128, 224), 1u);
-                            } else {  // d = 7 is new here, d = 1..6 are not
+#pragma unroll
+                                for (int p = kDigits - 1; p >= 1; --p)
+                                    ptx::mma_bf16(d + 32u * p, da + ((p * kASlice) >> 4), db,
+                                                  ptx::idesc_bf16_f32(128, 32 * (8 - p)), 1u);
+                                ptx::mma_bf16(d, da, db, ptx::idesc_bf16_f32(128, 224), 1u);
+                            } else {  // d = 0..6 are new with digit 0, d = 7 with digit 1
+                                ptx::mma_bf16(d, da, db, ptx::idesc_bf16_f32(128, 224), 0u);
                                 ptx::mma_bf16(d + 32u, da + (kASlice >> 4), db,
                                               ptx::idesc_bf16_f32(128, 192), 1u);
                                 ptx::mma_bf16(d + 224u, da + (kASlice >> 4),
                                               db + ((6 * kBSlice) >> 4),
                                               ptx::idesc_bf16_f32(128, 32), 0u);
-                            }
 #pragma unroll
-                            for (int p = 2; p < kDigits; ++p)
-                                ptx::mma_bf16(d + 32u * p, da + ((p * kASlice) >> 4), db,
-                                              ptx::idesc_bf16_f32(128, 32 * (8 - p)), 1u);
+                                for (int p = kDigits - 1; p >= 2; --p)
+                                    ptx::mma_bf16(d + 32u * p, da + ((p * kASlice) >> 4), db,
+                                                  ptx::idesc_bf16_f32(128, 32 * (8 - p)), 1u);
+                            }
                             if (sub == 1) ptx::mma_commit(ptx::smem_u32(&empty[stage]));
                             if (++stage == kStages) {
                                 stage = 0;
@@ -317,28 +322,27 @@ __global__ void __launch_bounds__(kThreads, 1)
             // partner lane holds the other of (Re, Im) of the same mode
             const int f = row_exp[tl.mt * 128 + row] - 70;
             const bool odd = (lane & 1) != 0;
-            double v[32];
+            // even lanes (Re rows) form the real parts ar br + ai bi, odd lanes
+            // the imaginary parts ai br - ar bi
+            const int64_t e0 = (int64_t)tl.st * 32 + sub * 16;
+            double v[16];
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
                 const double a = fixed_to_double(hi[c], lo[c], f);
                 const double b = fixed_to_double(hi[16 + c], lo[16 + c], f);
+                const double pa = __shfl_xor_sync(0xffffffffu, a, 1);
                 const double pb = __shfl_xor_sync(0xffffffffu, b, 1);
-                v[c] = a * b;                       // ar br, ai bi
-                v[16 + c] = odd ? a * pb : -(a * pb);  // ai br, -ar bi
+                v[c] = fma(a, odd ? pb : b, odd ? -(pa * b) : pa * pb);
             }
             if (occ.p) {
                 const int mode = tl.mt * 64 + (row >> 1);
                 double *dst = occ.p + (size_t)mode * occ.ld + (odd ? occ.plane : 0);
-                const int64_t e0 = (int64_t)tl.st * 32 + sub * 16;
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const double re = v[c] + __shfl_xor_sync(0xffffffffu, v[c], 1);
-                    const double im = v[16 + c] + __shfl_xor_sync(0xffffffffu, v[16 + c], 1);
-                    if (e0 + c < count) dst[e0 + c] = odd ? im : re;
-                }
+                for (int c = 0; c < 16; ++c)
+                    if (e0 + c < count) dst[e0 + c] = v[c];
             }
             const double s = transpose_sum(v, lane);
-            red[(quarter * 2 + sub) * 32 + lane] = s;
+            red[(quarter * 2 + sub) * 32 + (odd ? 16 : 0) + (lane >> 1)] = s;
             // the four lane quarters of this sub-tile
             asm volatile("bar.sync %0, 128;" ::"r"(1 + sub) : "memory");
             if (quarter == 0 && lane < 16) {
@@ -348,8 +352,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     re += red[(q * 2 + sub) * 32 + lane];
                     im += red[(q * 2 + sub) * 32 + 16 + lane];
                 }
-                const int64_t e = (int64_t)tl.st * 32 + sub * 16 + lane;
-                if (e < count) nS_part[(size_t)tl.mt * ld_part + e] = make_double2(re, im);
+                if (e0 + lane < count) nS_part[(size_t)tl.mt * ld_part + e0 + lane] = make_double2(re, im);
             }
             asm volatile("bar.sync %0, 128;" ::"r"(1 + sub) : "memory");
         }
