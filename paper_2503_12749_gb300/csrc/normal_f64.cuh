@@ -137,8 +137,7 @@ __device__ __forceinline__ void normals(uint32_t c0, uint32_t c1, uint32_t c2, u
     q = df_add_f(q, -1.0f);
     const df corr = df_mul(df_mul(r, r), q);
     const df sm = df_add_f(df_neg(corr), g.lo + k.lo);
-    // the small parts first (their roundings lie below 2^-62): one rounding of W
-    const double W = (k.hi + g.hi) + ((f2d(sm.hi) + f2d(sm.lo)) - r2d);
+    const double W = ((k.hi + g.hi) - r2d) + (f2d(sm.hi) + f2d(sm.lo));
     // ---- rho = sqrt(W)
     const df wd = d2df(W);
     const float y = rsqrtf(wd.hi);
