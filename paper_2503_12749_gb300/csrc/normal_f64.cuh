@@ -8,9 +8,9 @@
 // polishes the root: 17 FP64 instructions per pair, samples included.  Measured
 // (ms, with the samples' stores): N = 1000, 32768 trajectories as digit tiles
 // 5.08 -> 1.13, N = 700, 20001 as FP32 tiles 2.60 -> 0.60, N = 16, 16384 0.116 ->
-// 0.028.  Errors against 113-bit arithmetic, relative to the radius, 4e5 random
-// pairs: root mean square 5.93e-17, largest 3.21e-16 (log, sqrt and sincospi: 5.92e-17,
-// 3.13e-16).
+// 0.028.  Errors against 113-bit arithmetic, relative to the radius, 1e6 random
+// pairs: root mean square 5.69e-17, largest 3.12e-16 (log, sqrt and sincospi: 5.93e-17,
+// 3.12e-16).
 //   -2 ln u:  u = m 2^E, t = round(4096 / centre of m's 1/512 interval),
 //             r = m t / 4096 - 1 exactly (64-bit integers, |r| < 2^-9.6),
 //             -2 ln u = -2 E ln 2 + 2 ln(t / 4096) - 2 ln(1 + r)
@@ -137,7 +137,8 @@ __device__ __forceinline__ void normals(uint32_t c0, uint32_t c1, uint32_t c2, u
     q = df_add_f(q, -1.0f);
     const df corr = df_mul(df_mul(r, r), q);
     const df sm = df_add_f(df_neg(corr), g.lo + k.lo);
-    const double W = ((k.hi + g.hi) - r2d) + (f2d(sm.hi) + f2d(sm.lo));
+    // the small parts first (their roundings lie below 2^-62): one rounding of W
+    const double W = (k.hi + g.hi) + ((f2d(sm.hi) + f2d(sm.lo)) - r2d);
     // ---- rho = sqrt(W)
     const df wd = d2df(W);
     const float y = rsqrtf(wd.hi);
