@@ -67,10 +67,13 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
 // lanes per SM and clock), so the transcendental part is spread over blocks of
 // 512 parameters (one block per network left an 8000-mode network on one SM),
 // with sinh from one expm1 (sinh r = (u + u / (u + 1)) / 2, u = e^r - 1) and cosh
-// 2r = 1 + 2 sinh^2 r.  One pass over r, which may lie in host memory: the
-// deviation is summed about the network's first parameter c (r varies about c
-// by the deviation itself, so nothing cancels beyond a few bits).
-// part[net][chunk] = sum r - c, sum (r - c)^2, sum sinh^2, sum sinh^4, min, max.
+// 2r = 1 + 2 sinh^2 r.  One pass over r, which may lie in host memory: sums of
+// r - c, c the network's first parameter, and squared deviations about each
+// block's own mean, which k_sur_features joins (Chan, Golub, LeVeque, "Algorithms
+// for computing the sample variance", Amer. Statist. 37, 1983): nothing cancels,
+// whatever c is.
+// part[net][chunk] = sum r - c, sum (r - c - its chunk mean)^2, sum sinh^2,
+// sum sinh^4, min, max.
 constexpr int kFeatChunk = 512;
 constexpr int kFeatPart = 6;
 
@@ -90,6 +93,7 @@ __global__ void __launch_bounds__(256) k_sur_feature_parts(const NetIn *__restri
         a[4] = fmin(a[4], b[4]);
         a[5] = fmax(a[5], b[5]);
     };
+    double dev[kFeatChunk / 256] = {};
 #pragma unroll
     for (int t = 0; t < kFeatChunk / 256; ++t) {
         const int j = j0 + t * 256 + threadIdx.x;
@@ -98,7 +102,8 @@ __global__ void __launch_bounds__(256) k_sur_feature_parts(const NetIn *__restri
         const double u = expm1(x);
         const double sh = 0.5 * (u + (u < 0x1p60 ? u / (u + 1.0) : 1.0));
         const double sh2 = sh * sh;
-        join(v, {x - c, (x - c) * (x - c), sh2, sh2 * sh2, x, x});
+        dev[t] = x - c;
+        join(v, {dev[t], 0.0, sh2, sh2 * sh2, x, x});
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -111,7 +116,20 @@ __global__ void __launch_bounds__(256) k_sur_feature_parts(const NetIn *__restri
 #pragma unroll
         for (int q = 0; q < kFeatPart; ++q) red[threadIdx.x >> 5][q] = v[q];
     __syncthreads();
+    double mean = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) mean += red[w][0];
+    mean /= (double)min(kFeatChunk, n.N - j0);
+    double m2 = 0.0;
+#pragma unroll
+    for (int t = 0; t < kFeatChunk / 256; ++t)
+        if (j0 + t * 256 + (int)threadIdx.x < n.N) m2 += (dev[t] - mean) * (dev[t] - mean);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][1] = m2;
+    __syncthreads();
     if (threadIdx.x == 0) {
+        v[1] = m2;
         for (int w = 1; w < 8; ++w) join(v, red[w]);
         double *o = part + ((size_t)blockIdx.y * chunks + blockIdx.x) * kFeatPart;
 #pragma unroll
@@ -143,6 +161,15 @@ __global__ void k_sur_features(const NetIn *__restrict__ nets, const double *__r
     // sum of eta sinh^2 + eta^2 sinh^2 (1 + 2 sinh^2)
     const double s = sqrt(mu + eta * mu + 2.0 * eta * eta * t[3]);
     const double d = t[0] / (double)n.N;
+    // the chunk means' own deviations, a chunk per lane
+    double between = 0.0;
+    for (int c = lane; c * kFeatChunk < n.N; c += 32) {
+        const double cnt = (double)min(kFeatChunk, n.N - c * kFeatChunk);
+        const double e = part[((size_t)i * chunks + c) * kFeatPart] / cnt - d;
+        between += cnt * e * e;
+    }
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) between += __shfl_xor_sync(0xffffffffu, between, w);
     double *o = rec + (size_t)i * kRec;
     // the logarithms side by side in the lanes
     double x = 1.0;
@@ -153,7 +180,7 @@ __global__ void k_sur_features(const NetIn *__restrict__ nets, const double *__r
     const double lg = log(x);
     if (lane == 0 || lane == 1 || lane == 8 || lane == 9) o[lane] = lg;
     if (lane == 2) o[2] = r[n.r0] + d;
-    if (lane == 3) o[3] = sqrt(fmax(t[1] / (double)n.N - d * d, 0.0));
+    if (lane == 3) o[3] = sqrt((t[1] + between) / (double)n.N);
     if (lane == 4) o[4] = t[4];
     if (lane == 5) o[5] = t[5];
     if (lane == 6) o[6] = n.t;
