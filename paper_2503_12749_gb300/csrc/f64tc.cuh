@@ -3,6 +3,8 @@
 // operand.
 #pragma once
 
+#include <cuda_fp16.h>
+
 #include <cstdint>
 
 namespace gbs {
@@ -40,16 +42,26 @@ __device__ __forceinline__ int64_t to_fixed(double v, int s) {
     return bits < 0 ? -x : x;
 }
 
-// The seven balanced digits of x (|x| <= 2^55) as BF16 bits, most significant
-// first: bytes of x + 128 (1 + 256 + ...), less 128.
-__device__ __forceinline__ void digits_bf16(int64_t x, uint16_t (&d)[kDigits]) {
-    const int64_t y = x + 0x808080808080ll;
-    d[0] = (uint16_t)(__float_as_uint((float)(int)(y >> 48)) >> 16);
+// The seven balanced digits of x0 and x1 (|x| <= 2^55) as pairs of FP16 numbers
+// (x0's in the low half), most significant first: bytes of x + 128 (1 + 256 +
+// ...), less 128.  FP16 rather than BF16 because a byte below 1024 is exact in
+// it, so both digits of a pair take one byte permutation, one logic instruction
+// and one packed subtraction.  The leading digit has 9 bits (0..256).
+__device__ __forceinline__ void digit_pairs(int64_t x0, int64_t x1, uint32_t (&d)[kDigits]) {
+    const uint64_t y0 = (uint64_t)x0 + 0x80808080808080ull, y1 = (uint64_t)x1 + 0x80808080808080ull;
+    const __half2 bias = __float2half2_rn(1152.0f);  // 1024 + 128
+    auto less = [&](uint32_t v) {
+        const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&v), bias);
+        return *reinterpret_cast<const uint32_t *>(&h);
+    };
+    const uint32_t h0 = (uint32_t)(y0 >> 32), h1 = (uint32_t)(y1 >> 32);
+    d[0] = less(__byte_perm(h0, h1, 0x7632) + 0x64006400u);
 #pragma unroll
     for (int q = 1; q < kDigits; ++q) {
-        const uint32_t b = (uint32_t)(y >> (8 * (kDigits - 1 - q))) & 255u;
-        // 2^23 + b, less 2^23 + 128: exact
-        d[q] = (uint16_t)(__float_as_uint(__uint_as_float(0x4B000000u | b) - 8388736.0f) >> 16);
+        const int byte = kDigits - 1 - q;
+        const uint32_t v = byte >= 4 ? __byte_perm(h0, h1, (byte - 4) | byte << 8)
+                                     : __byte_perm((uint32_t)y0, (uint32_t)y1, byte | (byte + 4) << 8);
+        d[q] = less((v & 0x00ff00ffu) | 0x64006400u);
     }
 }
 

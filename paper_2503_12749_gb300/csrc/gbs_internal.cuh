@@ -49,7 +49,7 @@ constexpr int kFp32TileSamples = 64;            // samples per FP32 GEMM tile
 constexpr int kFp32BlockK = 16;                 // input modes per FP32 GEMM stage
 // Input modes from which the FP64 GEMM runs as digit products on the tensor
 // cores (k_gemm_f64tc.cu): one whole K step.  It is the faster one at every
-// size (N = M = 16, 16384 trajectories: 0.054 against 0.150 ms), but its
+// size (N = M = 16, 16384 trajectories: 0.049 against 0.150 ms), but its
 // error grows as sqrt(N) against the FMA chain's N, and below about 10 modes
 // the chain's is the smaller.
 constexpr int kF64tcMinN = 16;

@@ -3,7 +3,7 @@
 // fused with the FP64 occupation epilogue n'_i = alpha'_i beta'_i.
 //
 // Both operands are written as fixed-point numbers of seven balanced 8-bit
-// digits and the digit products are contracted without rounding on the BF16
+// digits and the digit products are contracted without rounding on the FP16
 // tensor cores (the error-free splitting of Ozaki, Ogita, Oishi, Rump,
 // "Error-free transformations of matrix multiplication by using fast routines
 // of matrix multiplication and its applications", Numer. Algorithms 59, 2012,
@@ -14,7 +14,7 @@
 //   alpha'_i = 2^{f_i - 70} sum_d D_d 2^{8 (7 - d)}.
 // e_j bounds |alpha_j|, |beta_j| for every possible draw (the Box-Muller
 // radius of a 53-bit uniform is below 8.67), f_i bounds row i of T 2^{e_j}.
-// A digit is an integer of at most 8 bits, so it is a BF16 number; 8 products
+// A digit is an integer of at most 8 bits, so it is an FP16 number; 8 products
 // of at most 2^14 over 128 input modes sum to at most 2^24, so every FP32
 // accumulator value is an exact integer.  The accumulators are added to
 // 64-bit integers every 128 modes, so the only errors are the quantisation
@@ -23,10 +23,11 @@
 // term against 0.6 N 2^-54 for a chain of FP64 FMAs.
 //
 // Why: GB300 has 2 FP64 FMA lanes per SM and clock (1.25 TFLOP/s) but 4096
-// BF16 ones, so 34 exact BF16 products cost a fiftieth of one FP64 product.
-// Measured (one GB300): N = M = 1000, 32768 trajectories 6.27 ms against 216.4
-// for the FP64 FMA kernel (34 products at 0.60 of the tensor pipe's rate);
-// N = M = 16, 16384 trajectories 0.054 against 0.150.  Root mean square error of
+// 16-bit ones, so 34 exact 16-bit products cost a fiftieth of one FP64 product.
+// Measured (one GB300): N = M = 1000, 32768 trajectories 5.50 ms against 216.4
+// for the FP64 FMA kernel (34 products at 0.84 of the measured BF16 rate; 6.27 with
+// a conversion for every sum and 32 columns read at once, f64tc_pipe.cuh);
+// N = M = 16, 16384 trajectories 0.049 against 0.150.  Root mean square error of
 // n_S against 113-bit arithmetic, relative to sum |alpha'_i| |beta'_i|:
 // N = 1000 1.9e-16 against 3.2e-16, N = 300 2.5e-16 against 3.1e-16, N = 64
 // 1.1e-16 against 1.3e-16, N = 16 3.1e-16 against 3.8e-16 (the input samples'
@@ -43,8 +44,7 @@
 // Operands are stored in global memory as the exact shared-memory images
 // (no swizzle, 8 x 16-byte core matrices), so a stage is two plain bulk copies.
 #include "gbs_internal.cuh"
-#include "f64tc.cuh"
-#include "tc_ptx.cuh"
+#include "f64tc_pipe.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -55,56 +55,12 @@ namespace {
 
 using namespace f64tc;
 
-constexpr int kStageBytes = kAStage + kBStage;
-constexpr int kStages = 5;    // 215 KB of the 227 KB
-constexpr int kBurst = 4;     // stages per sub-tile turn
-constexpr int kChunkKB = 8;   // K blocks (of 16) per exact accumulation: 128 modes
-constexpr int kEpiWarps = 8;  // 4 lane quarters x 2 sub-tiles
-constexpr int kThreads = 64 + 32 * kEpiWarps;
-constexpr int kBarBytes = 256;
 constexpr int kRedBytes = 4 * 2 * 32 * 8;  // [quarter][sub-tile][16 re, 16 im]
-constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kBarBytes + kRedBytes;
+constexpr int kSmemBytes = kPipeBytes + kRedBytes;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory of the FP64 tensor-core GEMM");
-static_assert(kChunkKB == 2 * kBurst, "a chunk is two turns of each sub-tile");
-// bound of every pipeline wait (gbs_set_wait_limit is for the BF16 paths)
-constexpr uint64_t kWaitNs = 2000000000ull;
 // mode tiles per band of the tile order: 8 mode tiles x 19 trajectory tiles
 // make one wave of 152 CTAs, the most square split of its operand traffic
 constexpr int kBand = 8;
-
-// K-major operand without swizzle: core matrices of 8 rows x 16 bytes; the
-// two of a 16-wide K step 128 bytes apart (leading offset), 8-row groups 256
-// bytes apart (stride offset); descriptor version 1 (bit 46).
-__device__ __forceinline__ uint64_t desc_k_plain(uint32_t saddr) {
-    return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)(128u >> 4) << 16 |
-           (uint64_t)(256u >> 4) << 32 | (uint64_t)1u << 46;
-}
-
-// (hi 2^32 + lo) 2^e as a double, rounded to nearest (integer instructions:
-// the FP64 pipe converts at 2 lanes per clock).
-__device__ __forceinline__ double fixed_to_double(int64_t hi, int64_t lo, int e) {
-    hi += lo >> 32;
-    uint32_t l = (uint32_t)lo;
-    const bool neg = hi < 0;
-    uint64_t h = (uint64_t)hi;
-    if (neg) {
-        l = 0u - l;
-        h = ~h + (l == 0u ? 1u : 0u);
-    }
-    if (h == 0) {
-        if (l == 0u) return 0.0;
-        h = l;
-        l = 0u;
-        e -= 32;
-    }
-    const int s = __clzll((long long)h);
-    const uint64_t m = (h << s) | ((((uint64_t)l << 32) >> 1) >> (63 - s));
-    const uint64_t r = (m >> 11) + ((m >> 10) & 1u);  // 53 bits, the top one set
-    // m 2^(e + 32 - s): its leading bit weighs 2^(63 + 32 - s + e)
-    const int64_t expo = (int64_t)(63 + 32 - s + e + 1023 - 1);
-    const int64_t bits = (expo << 52) + (int64_t)r;
-    return __longlong_as_double(bits | (neg ? (int64_t)0x8000000000000000ull : 0));
-}
 
 struct Tile {
     int mt, st;
@@ -141,150 +97,26 @@ __global__ void __launch_bounds__(kThreads, 1)
                  int64_t count, int64_t ld_part, double2 *__restrict__ nS_part, OccOut64 occ,
                  uint64_t wait_ns, unsigned long long *err_ptr) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);
-    uint64_t *full = bars, *empty = bars + kStages;
-    uint64_t *tfull = bars + 2 * kStages, *tempty = tfull + 2;
-    uint64_t *drain = tempty + 2;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
-    double *red = reinterpret_cast<double *>(smem + kStages * kStageBytes + kBarBytes);
-
+    Pipe pipe(smem_raw);
+    double *red = reinterpret_cast<double *>(pipe.rest(smem_raw));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile unsigned long long *err = err_ptr;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
-            ptx::mbar_init(ptx::smem_u32(&full[s]), 1);
-            ptx::mbar_init(ptx::smem_u32(&empty[s]), 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(ptx::smem_u32(&tfull[b]), 1);
-            ptx::mbar_init(ptx::smem_u32(&tempty[b]), kEpiWarps / 2);
-        }
-        ptx::mbar_init(ptx::smem_u32(drain), 1);
-        ptx::fence_barrier_init();
-    }
-    if (warp == 1) {
-        ptx::tmem_alloc<1>(ptx::smem_u32(tmem_slot), 512);
-        ptx::tmem_relinquish<1>();
-    }
-    ptx::tc_fence_before();
-    __syncthreads();
-    ptx::tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = pipe.open();
     const int ntiles = mtiles * stiles;
     const int nchunk = (KB + kChunkKB - 1) / kChunkKB;
 
+    auto job = [&](int i, Contraction &c) {
+        const int64_t t = blockIdx.x + (int64_t)i * gridDim.x;
+        if (t >= ntiles) return false;
+        const Tile tl = tile_of((int)t, mtiles, stiles);
+        c = {A + (size_t)tl.mt * KB * kAStage, B + (size_t)tl.st * KB * kBStage, kAStage, kBStage, KB};
+        return true;
+    };
+
     if (warp == 0) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0, used = 0, last = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x) {
-                const Tile tl = tile_of(t, mtiles, stiles);
-                const uint8_t *a = A + (size_t)tl.mt * KB * kAStage;
-                const uint8_t *b = B + (size_t)tl.st * KB * kBStage;
-                for (int kb = 0; kb < KB; ++kb) {
-                    if (!ptx::mbar_wait(ptx::smem_u32(&empty[stage]), phase ^ 1u, err, wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t fb = ptx::smem_u32(&full[stage]);
-                    uint8_t *s = smem + stage * kStageBytes;
-                    ptx::mbar_arrive_expect_tx(fb, kStageBytes);
-                    ptx::bulk_load(ptx::smem_u32(s), a + (size_t)kb * kAStage, kAStage, fb);
-                    ptx::bulk_load(ptx::smem_u32(s + kAStage), b + (size_t)kb * kBStage, kBStage, fb);
-                    used |= 1u << stage;
-                    last = (last & ~(1u << stage)) | (phase << stage);
-                    if (++stage == kStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                }
-            }
-            // every load issued here has landed before the CTA exits
-            for (int s = 0; s < kStages; ++s)
-                if (used & (1u << s))
-                    ptx::mbar_wait(ptx::smem_u32(&full[s]), (last >> s) & 1u, err, 200000000ull,
-                                   false);
-        }
+        if (lane == 0) pipe.load(job, err, wait_ns);
     } else if (warp == 1) {
-        if (lane == 0) {
-            int base = 0;         // ring stage of the turn's first K block
-            uint32_t base_ph = 0; // its phase
-            uint32_t ck = 0;      // chunks issued so far
-            bool ok = true;
-            for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x) {
-                for (int kb0 = 0; ok && kb0 < KB; kb0 += kBurst) {
-                    const int nb = min(kBurst, KB - kb0);
-                    const bool first = kb0 % kChunkKB == 0;
-                    const bool end = !first || kb0 + nb >= KB;  // the chunk's last turn
-                    for (int sub = 0; ok && sub < 2; ++sub) {
-                        if (first) {
-                            // the epilogue has read the sub-tile's previous chunk
-                            if (!ptx::mbar_wait(ptx::smem_u32(&tempty[sub]), (ck & 1u) ^ 1u, err,
-                                                wait_ns)) {
-                                ok = false;
-                                break;
-                            }
-                            ptx::tc_fence_after();
-                        }
-                        int stage = base;
-                        uint32_t ph = base_ph;
-                        for (int q = 0; q < nb; ++q) {
-                            if (sub == 0) {
-                                if (!ptx::mbar_wait(ptx::smem_u32(&full[stage]), ph, err, wait_ns)) {
-                                    ok = false;
-                                    break;
-                                }
-                                ptx::tc_fence_after();
-                            }
-                            const uint8_t *s = smem + stage * kStageBytes;
-                            const uint64_t da = desc_k_plain(ptx::smem_u32(s));
-                            const uint64_t db =
-                                desc_k_plain(ptx::smem_u32(s + kAStage + sub * kBSub));
-                            const uint32_t d = tmem + (uint32_t)sub * 256u;
-                            const uint32_t acc = (first && q == 0) ? 0u : 1u;
-                            // digit p of A against digits 0..min(6, 7 - p) of B; the
-                            // long products last, so that the pipe has work while
-                            // the next stage's barrier is polled
-                            if (acc) {
-#pragma unroll
-                                for (int p = kDigits - 1; p >= 1; --p)
-                                    ptx::mma_bf16(d + 32u * p, da + ((p * kASlice) >> 4), db,
-                                                  ptx::idesc_bf16_f32(128, 32 * (8 - p)), 1u);
-                                ptx::mma_bf16(d, da, db, ptx::idesc_bf16_f32(128, 224), 1u);
-                            } else {  // d = 0..6 are new with digit 0, d = 7 with digit 1
-                                ptx::mma_bf16(d, da, db, ptx::idesc_bf16_f32(128, 224), 0u);
-                                ptx::mma_bf16(d + 32u, da + (kASlice >> 4), db,
-                                              ptx::idesc_bf16_f32(128, 192), 1u);
-                                ptx::mma_bf16(d + 224u, da + (kASlice >> 4),
-                                              db + ((6 * kBSlice) >> 4),
-                                              ptx::idesc_bf16_f32(128, 32), 0u);
-#pragma unroll
-                                for (int p = kDigits - 1; p >= 2; --p)
-                                    ptx::mma_bf16(d + 32u * p, da + ((p * kASlice) >> 4), db,
-                                                  ptx::idesc_bf16_f32(128, 32 * (8 - p)), 1u);
-                            }
-                            if (sub == 1) ptx::mma_commit(ptx::smem_u32(&empty[stage]));
-                            if (++stage == kStages) {
-                                stage = 0;
-                                ph ^= 1u;
-                            }
-                        }
-                        if (!ok) break;
-                        if (end) ptx::mma_commit(ptx::smem_u32(&tfull[sub]));
-                        if (sub == 1) {
-                            base = stage;
-                            base_ph = ph;
-                        }
-                    }
-                    if (end) ++ck;
-                }
-            }
-            ptx::mma_commit(ptx::smem_u32(drain));
-            ptx::mbar_wait(ptx::smem_u32(drain), 0u, err, 200000000ull, false);
-        }
+        if (lane == 0) pipe.multiply(job, tmem, err, wait_ns);
     } else {
         const int quarter = warp & 3;
         const int sub = (warp - 2) >> 2;
@@ -293,31 +125,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t ck = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
             const Tile tl = tile_of(t, mtiles, stiles);
-            int64_t hi[32], lo[32];  // sum_{d < 4} D_d 2^{8 (3 - d)}, sum_{d >= 4} D_d 2^{8 (7 - d)}
+            int64_t hi[32], lo[32];
 #pragma unroll
             for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
-            for (int k = 0; k < nchunk; ++k, ++ck) {
-                // on a timeout the epilogue keeps going without waiting
-                ptx::mbar_wait(ptx::smem_u32(&tfull[sub]), ck & 1u, err, wait_ns);
-                ptx::tc_fence_after();
-#pragma unroll
-                for (int d = 0; d < 8; ++d) {
-                    float v[32];
-                    ptx::tmem_ld32(tb + 32u * d, v);
-                    ptx::tmem_ld_wait();
-                    if (d == 7) {
-                        ptx::tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&tempty[sub]));
-                    }
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        const int64_t x = (int64_t)__float2int_rn(v[c]) * (1 << (8 * (3 - (d & 3))));
-                        if (d < 4) hi[c] += x;
-                        else lo[c] += x;
-                    }
-                }
-            }
+            for (int k = 0; k < nchunk; ++k, ++ck) pipe.add_chunk(ck, sub, tb, hi, lo, err, wait_ns);
             // alpha' (columns 0..15) and beta' (16..31) of this row; the
             // partner lane holds the other of (Re, Im) of the same mode
             const int f = row_exp[tl.mt * 128 + row] - 70;
@@ -357,10 +168,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             asm volatile("bar.sync %0, 128;" ::"r"(1 + sub) : "memory");
         }
     }
-    ptx::tc_fence_before();
-    __syncthreads();
-    ptx::tc_fence_after();
-    if (warp == 1) ptx::tmem_dealloc<1>(tmem, 512);
+    pipe.close(tmem);
 }
 
 // One block per row (mode i, Re or Im) of the padded operand: the row's
@@ -400,11 +208,11 @@ __global__ void __launch_bounds__(256) k_f64tc_split_T(const double *__restrict_
             const double v = src[j];
             if (v != 0.0) x = to_fixed(v, 55 + col_exp[j] - ex);
         }
-        uint16_t dg[kDigits];
-        digits_bf16(x, dg);
+        uint32_t dg[kDigits];
+        digit_pairs(x, 0, dg);
         uint8_t *p = tile + (size_t)(j >> 4) * kAStage + core_offset(r, j & 15);
 #pragma unroll
-        for (int q = 0; q < kDigits; ++q) *reinterpret_cast<uint16_t *>(p + q * kASlice) = dg[q];
+        for (int q = 0; q < kDigits; ++q) *reinterpret_cast<uint16_t *>(p + q * kASlice) = (uint16_t)dg[q];
     }
 }
 

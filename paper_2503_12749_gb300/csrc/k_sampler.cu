@@ -148,26 +148,27 @@ __global__ void __launch_bounds__(256, 2)
             for (int oct = (warp & (wpg - 1)) * 4 + (lane >> 3); oct < 2 * KB; oct += 4 * wpg) {
                 uint32_t da[kDigits][4], db[kDigits][4];
 #pragma unroll
-                for (int q = 0; q < kDigits; ++q)
+                for (int t = 0; t < 8; t += 2) {
+                    int64_t xa[2] = {0, 0}, xb[2] = {0, 0};
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) da[q][t] = db[q][t] = 0u;
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const int j = oct * 8 + t;
-                    if (j < N) {
-                        double a, b;
-                        amplitudes(sh, seed, e, (uint32_t)j, sq[j], a, b);
-                        part = fma(a, b, part);
-                        const int s = 55 - col_exp[j];
-                        uint16_t pa[kDigits], pb[kDigits];
-                        digits_bf16(to_fixed(a, s), pa);
-                        digits_bf16(to_fixed(b, s), pb);
-#pragma unroll
-                        for (int q = 0; q < kDigits; ++q) {
-                            da[q][t >> 1] |= (uint32_t)pa[q] << (16 * (t & 1));
-                            db[q][t >> 1] |= (uint32_t)pb[q] << (16 * (t & 1));
+                    for (int h = 0; h < 2; ++h) {
+                        const int j = oct * 8 + t + h;
+                        if (j < N) {
+                            double a, b;
+                            amplitudes(sh, seed, e, (uint32_t)j, sq[j], a, b);
+                            part = fma(a, b, part);
+                            const int s = 55 - col_exp[j];
+                            xa[h] = to_fixed(a, s);
+                            xb[h] = to_fixed(b, s);
                         }
                     }
+                    uint32_t w[kDigits];
+                    digit_pairs(xa[0], xa[1], w);
+#pragma unroll
+                    for (int q = 0; q < kDigits; ++q) da[q][t >> 1] = w[q];
+                    digit_pairs(xb[0], xb[1], w);
+#pragma unroll
+                    for (int q = 0; q < kDigits; ++q) db[q][t >> 1] = w[q];
                 }
                 uint8_t *p = tile + (size_t)(oct >> 1) * kBStage;
                 const int k = (oct & 1) * 8;
