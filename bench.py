@@ -85,15 +85,18 @@ GF_FP32_OPS_PER_PAIR = 200.5
 # FP64 peak: the FMA-chain probe (gbs_measure_fp64_rate, CUDA events; 8 to
 # 32 independent chains per thread, 128 to 1024 threads per block, 1 to 8
 # blocks per SM, outer-product and recurrence operand patterns) tops out at
-# 1.057 TFLOP/s on GB300, below the 1.25 the FP64 GEMM itself sustains on
-# m8000 (8MN FLOP per trajectory over CUDA-event kernel time), so the
-# larger of the probe and GB300's nominal FP64 rate is the peak.
+# 1.057 TFLOP/s on GB300, below the 1.25 a plain FP64 GEMM (k_gemm_fp64)
+# sustains on m8000 (8MN FLOP per trajectory over CUDA-event kernel time), so
+# the larger of the probe and GB300's nominal FP64 rate is the FP64 pipe's peak.
+# The FP64 path's GEMM (k_gemm_f64tc) forms its products as 34 exact digit
+# products on the tensor cores and exceeds it.
+F64TC_PRODUCTS = 34
 FP64_NOMINAL_TFLOPS = 1.25
 # FP32 FMA peak from unit counts: 152 SMs x 128 FP32 lanes x 2 FLOP x 2.07 GHz
 FP32_UNIT_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 FP32_PEAK_SOURCE = "unit counts: 152 SMs x 128 FP32 lanes x 2 FLOP per FMA x 2.07 GHz (maximum clock)"
 FP64_PEAK_SOURCE = ("max(gbs_measure_fp64_rate, nominal GB300 FP64 1.25 TFLOP/s): the "
-                    "FMA-chain probe reads below the rate the FP64 GEMM sustains")
+                    "FMA-chain probe reads below the rate a plain FP64 GEMM sustains")
 
 
 def _env_int(name, default):
@@ -434,15 +437,16 @@ def gbs_arm(args, wl_def):
         achieved = flops / (gemm_ms / 1e3) / 1e12
         peak = FP32_UNIT_TFLOPS
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak, "traffic": None, "kernel": "k_gemm_fp64<float>",
+                "frac": achieved / peak, "traffic": None, "kernel": "k_gemm_fp32",
                 "peak_source": FP32_PEAK_SOURCE}
     else:
         achieved = flops / (gemm_ms / 1e3) / 1e12
         probe = gbs.gbs_measure_fp64_rate(sptr)
         peak = max(probe, FP64_NOMINAL_TFLOPS)
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak if peak else None, "traffic": None,
-                "kernel": "k_gemm_fp64", "fp64_probe_tflops": probe,
+                "kernel": "k_gemm_f64tc", "fp64_probe_tflops": probe,
+                "digit_products_tflops": achieved * F64TC_PRODUCTS,
                 "peak_source": FP64_PEAK_SOURCE}
     phases = {k: {"ms_per_step": v[0] / args.steps, "launches_per_step": v[1] / args.steps}
               for k, v in prof.items()}
@@ -529,12 +533,14 @@ def gbs_arm(args, wl_def):
             "fp64_peak_tflops": fp64_peak, "fp64_probe_tflops": fp64_probe,
             "fp64_peak_source": FP64_PEAK_SOURCE,
             "gemm_frac_of_fp64_peak": fp64_gemm_tflops / fp64_peak if fp64_peak else None,
+            "gemm_digit_products_tflops": fp64_gemm_tflops * F64TC_PRODUCTS,
             "speedup_of_split_path": value / (Ef / (ms64 / 1e3)),
             "max_abs_dP_over_sigma_fp64": float(np.max(np.abs(Pb[0] - P64[0]) / sig)),
             "max_abs_dP_plusP_over_sigma_fp64": float(np.max(np.abs(Pb[2] - P64[2]) /
                                                              np.maximum(P64[3], 1e-13))),
             "what": f"gbs_sample of {Ef} trajectories on a GBS_FP64 network (FP64 sampler, "
-                    "SIMT FP64 GEMM, FP64 generating functions; CUDA events) and on a "
+                    "FP64 GEMM as exact digit products on the tensor cores, FP64 generating "
+                    "functions; CUDA events) and on a "
                     f"{precision} network, the same trajectories; speed-up = the timed "
                     "split-path value / this FP64 rate"}
 
@@ -779,10 +785,10 @@ def bin2d_arm(args):
                    "max_abs_P_odd_total": float(np.max(np.abs(
                        P[0][(np.add.outer(np.arange(K), np.arange(K)) % 2) == 1])))},
         "roofline": {"bound": "alu", "achieved": None, "peak": None, "unit": None,
-                     "frac": None, "traffic": None, "kernel": "k_gf2d_df",
-                     "note": "issue-bound double-float generating functions on the FP32 "
-                             "pipes, like the one-bin k_gf_df (see profiles/); not measured "
-                             "separately for this workload"},
+                     "frac": None, "traffic": None, "kernel": "k_sep_digits, k_gf2d_tc",
+                     "note": "double-float factors written as digits (bound by their "
+                             "instructions), contracted exactly on the tensor cores; not "
+                             "measured separately for this workload"},
         "phases": {k: {"ms": v[0], "launches": v[1]} for k, v in prof.items() if v[1]},
         "gpu_launches": launches_per_step * args.steps, "clocks": clk,
     }

@@ -276,4 +276,68 @@ __device__ __forceinline__ df2 df2_mul(df2 x, df2 y) {
     return df2_fast_two_sum(p, e);
 }
 
+// df_exp_tab and df_sincos_tab of two arguments side by side (per lane the same
+// operations).
+__device__ __forceinline__ df2 df2_exp_tab(df2 a, const DfTables &T, const DfConsts &K) {
+    const float2 kf = f2(rintf(a.hi.x * 92.33248261689366f), rintf(a.hi.y * 92.33248261689366f));
+    const float2 kn = f2_neg(kf);
+    df2 r = df2_two_sum(f2_fma(kn, f2(K.ln2_64_1, K.ln2_64_1), a.hi), a.lo);
+    r = df2_add_f(r, f2_mul(kn, f2(K.ln2_64_2, K.ln2_64_2)));
+    r = df2_add_f(r, f2_mul(kn, f2(K.ln2_64_3, K.ln2_64_3)));
+    const float2 x = r.hi;
+    const float2 qt = f2_mul(x, f2_fma(f2_fma(x, f2(1.0f / 120.0f, 1.0f / 120.0f), f2(1.0f / 24.0f, 1.0f / 24.0f)),
+                                       x, f2(1.0f / 6.0f, 1.0f / 6.0f)));
+    const df2 q = df2_fast_two_sum(f2(0.5f, 0.5f), qt);
+    const df2 p = df2_add_f(df2_add(r, df2_mul(df2_mul(r, r), q)), f2(1.0f, 1.0f));
+    const int n0 = (int)kf.x, n1 = (int)kf.y;
+    const df2 t = df2_mul(df2_make(T.exp2[n0 & 63], T.exp2[n1 & 63]), p);
+    const float2 scale = f2(__int_as_float(((n0 >> 6) + 127) << 23), __int_as_float(((n1 >> 6) + 127) << 23));
+    return {f2_mul(t.hi, scale), f2_mul(t.lo, scale)};
+}
+
+__device__ __forceinline__ df2 df2_neg(df2 a) { return {f2_neg(a.hi), f2_neg(a.lo)}; }
+
+__device__ __forceinline__ void df2_sincos_tab(df2 phi, const DfTables &T, const DfConsts &K,
+                                               df2 &s_out, df2 &c_out) {
+    const float2 qf = f2(rintf(phi.hi.x * 0.636619772367581343076f), rintf(phi.hi.y * 0.636619772367581343076f));
+    const float2 qn = f2_neg(qf);
+    df2 s = df2_two_sum(f2_fma(qn, f2(K.pio2_1, K.pio2_1), phi.hi), phi.lo);
+    s = df2_add_f(s, f2_mul(qn, f2(K.pio2_2, K.pio2_2)));
+    s = df2_add_f(s, f2_mul(qn, f2(K.pio2_3, K.pio2_3)));
+    s = df2_add_f(s, f2_mul(qn, f2(K.pio2_4, K.pio2_4)));
+    const float2 jf = f2(fminf(fmaxf(rintf(s.hi.x * 20.371832715762604f), -16.0f), 16.0f),
+                         fminf(fmaxf(rintf(s.hi.y * 20.371832715762604f), -16.0f), 16.0f));
+    const float2 jn = f2_neg(jf);
+    df2 r = df2_two_sum(f2_fma(jn, f2(K.pi64_1, K.pi64_1), s.hi), s.lo);
+    r = df2_add_f(r, f2_mul(jn, f2(K.pi64_2, K.pi64_2)));
+    r = df2_add_f(r, f2_mul(jn, f2(K.pi64_3, K.pi64_3)));
+    const df2 r2 = df2_mul(r, r);
+    const float2 x = r2.hi, xx = f2_mul(x, x);
+    const float2 ts = f2_mul(xx, f2_fma(f2_neg(x), f2(1.0f / 5040.0f, 1.0f / 5040.0f),
+                                        f2(1.0f / 120.0f, 1.0f / 120.0f)));
+    const df2 sixth = {f2(-0x1.555556p-3f, -0x1.555556p-3f), f2(0x1.555556p-28f, 0x1.555556p-28f)};
+    const df2 sr = df2_mul(r, df2_add_f(df2_add_f(df2_mul(r2, sixth), ts), f2(1.0f, 1.0f)));
+    const float2 tc = f2_mul(xx, f2_fma(f2_fma(x, f2(1.0f / 40320.0f, 1.0f / 40320.0f),
+                                               f2(-1.0f / 720.0f, -1.0f / 720.0f)),
+                                        x, f2(1.0f / 24.0f, 1.0f / 24.0f)));
+    const float2 mh = f2(-0.5f, -0.5f);
+    const df2 cr = df2_add_f(df2_add_f(df2{f2_mul(mh, r2.hi), f2_mul(mh, r2.lo)}, tc), f2(1.0f, 1.0f));
+    const int j0 = (int)jf.x + 16, j1 = (int)jf.y + 16;
+    const df2 S = df2_make(T.sn[j0], T.sn[j1]), C = df2_make(T.cs[j0], T.cs[j1]);
+    const df2 sn = df2_add(df2_mul(S, cr), df2_mul(C, sr));
+    const df2 cs = df2_add(df2_mul(C, cr), df2_neg(df2_mul(S, sr)));
+    // quadrants: (s, c), (c, -s), (-s, -c), (-c, s)
+    auto turn = [](int q, float s0, float c0, float &so, float &co) {
+        const bool odd = (q & 1) != 0;
+        const float a = odd ? c0 : s0, b = odd ? s0 : c0;
+        so = __uint_as_float(__float_as_uint(a) ^ ((uint32_t)(q & 2) << 30));
+        co = __uint_as_float(__float_as_uint(b) ^ ((uint32_t)((q + 1) & 2) << 30));
+    };
+    const int q0 = (int)qf.x, q1 = (int)qf.y;
+    turn(q0, sn.hi.x, cs.hi.x, s_out.hi.x, c_out.hi.x);
+    turn(q0, sn.lo.x, cs.lo.x, s_out.lo.x, c_out.lo.x);
+    turn(q1, sn.hi.y, cs.hi.y, s_out.hi.y, c_out.hi.y);
+    turn(q1, sn.lo.y, cs.lo.y, s_out.lo.y, c_out.lo.y);
+}
+
 }  // namespace gbs

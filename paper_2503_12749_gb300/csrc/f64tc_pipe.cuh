@@ -1,7 +1,8 @@
 // The pipeline of the exact digit-product contractions (f64tc.cuh): bulk copies
 // of operand stages, the products of the digits into eight sums D_d per
-// sub-tile, and the barriers between them and the epilogue warps (the FP64 GEMM,
-// k_gemm_f64tc.cu).
+// sub-tile, and the barriers between them and the epilogue warps.  Used by the
+// FP64 GEMM (k_gemm_f64tc.cu) and the joint generating functions
+// (k_gf2d_tc.cu), which differ in what their operands are and where the sums go.
 #pragma once
 
 #include "f64tc.cuh"

@@ -191,6 +191,8 @@ void release_estimator(gbs_net *net) {
     net_free(net, net->d_out2);
     net_free(net, net->d_mo2);
     pool_free(net->d_sep2, net->stream);
+    pool_free(net->d_gf2, net->stream);
+    net->gf2_bytes = 0;
     net->counts2.clear();
     net->est2_fixed = false;
     net->n_sub2 = 0;
@@ -1231,8 +1233,9 @@ int gbs_sample_nd(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E
             if ((r = launch_finalize2d(net, c))) return r;
             prof_mark(net, GBS_PHASE_FINALIZE, 1, false);
             prof_mark(net, GBS_PHASE_GF, 0, true);
-            if ((r = launch_gf2d(net, e0, c))) return r;
-            prof_mark(net, GBS_PHASE_GF, 2, false);
+            int nl;
+            if ((r = launch_gf2d(net, e0, c, &nl))) return r;
+            prof_mark(net, GBS_PHASE_GF, nl, false);
             return GBS_OK;
         };
         if ((rc = pipelined_chunks(net, seed, first_sample, E, net->chunk, gemm, after))) return rc;
@@ -1242,8 +1245,9 @@ int gbs_sample_nd(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E
             const uint64_t e0 = first_sample + (uint64_t)done;
             if ((rc = run_chunk_front2d(net, seed, e0, c))) return rc;
             prof_mark(net, GBS_PHASE_GF, 0, true);
-            if ((rc = launch_gf2d(net, e0, c))) return rc;
-            prof_mark(net, GBS_PHASE_GF, simt_precision(net->precision) ? 1 : 2, false);
+            int nl;
+            if ((rc = launch_gf2d(net, e0, c, &nl))) return rc;
+            prof_mark(net, GBS_PHASE_GF, nl, false);
         }
     }
     const uint64_t ns = (uint64_t)net->n_sub2;

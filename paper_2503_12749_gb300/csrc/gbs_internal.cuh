@@ -253,6 +253,8 @@ struct gbs_net {
     double *d_out2 = nullptr;       // [4][grid2]
     int64_t *d_mo2 = nullptr;       // [kMaxBins] DFT window offsets
     void *d_sep2 = nullptr;         // [chunk] per-trajectory constants (BF16 networks)
+    void *d_gf2 = nullptr;          // work space of the digit-product kernels (k_gf2d_tc.cu)
+    size_t gf2_bytes = 0;
 };
 
 namespace gbs {
@@ -433,7 +435,7 @@ int launch_moment_stats(const MomentSpec &sp, bool fp64, const double *acc, cons
 // generating functions on the K_1 x .. x K_d grid, and the d-dimensional
 // inversion into out_dev[4][grid2] (*launches: kernels launched).
 int launch_finalize2d(gbs_net *net, int64_t count);
-int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count);
+int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count, int *launches);
 size_t sep2_bytes_per_trajectory();
 int launch_tables2d(gbs_net *net);
 int launch_invert2d(gbs_net *net, const int64_t *m_off, double *out_dev, int *launches);

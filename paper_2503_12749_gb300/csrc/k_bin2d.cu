@@ -24,25 +24,19 @@
 // likewise for the e^{-L} term around (pi, .., pi).  Sub-ensemble sums are
 // inverted by a d-dimensional FFT: per dimension, FFTs along the innermost
 // one and a rotation that moves it outermost.
-#include "gbs_internal.cuh"
-#include "dfloat.cuh"
+#include "bin2d.cuh"
 
+#include <algorithm>
 #include <cmath>
 
 namespace gbs {
 namespace {
 
+using namespace bin2d;
+
 constexpr double kTwoPi2 = 6.283185307179586476925286766559;
 constexpr int kG2Threads = 128;
 constexpr int kG2Tile = 128;
-
-// Shape of one launch over the grid (passed by value).
-struct GridD {
-    int d;                   // bins
-    int K[kMaxBins];         // points per dimension
-    int Koff[kMaxBins];      // offsets of each dimension's tables
-    int tile[kMaxBins + 1];  // bin b = GEMM tiles [tile[b], tile[b + 1])
-};
 
 // max over c in [0, 2] of -c x + sqrt(2c) |y|
 __device__ __forceinline__ double max_term1(double x, double y) {
@@ -146,67 +140,10 @@ __global__ void k_finalize2d(const double2 *__restrict__ part, const GridD g, in
         for (int q = 0; q < 2 * kMaxBins; ++q) atomicMax(&wmax[q], m[q]);
 }
 
-__device__ __forceinline__ int slots_of(int K, int W1, int W2) {
-    const int half = K >> 1;
-    const int n1 = W1 >= half ? K : 2 * W1 + 1;
-    const int n2 = W2 < 0 ? 0 : (W2 >= half ? K : 2 * W2 + 1);
-    return n1 + n2 >= K ? K : n1 + n2;
-}
-
-// k of slot i of one dimension: the window around 0 (k = -W1..W1), then the
-// one around K/2; the whole range when they cover it.
-__device__ __forceinline__ int slot_k(int i, int K, int W1, int W2) {
-    const int half = K >> 1;
-    const int n1 = W1 >= half ? K : 2 * W1 + 1;
-    const int n2 = W2 < 0 ? 0 : (W2 >= half ? K : 2 * W2 + 1);
-    if (n1 + n2 >= K) return i;
-    if (i < n1) {
-        const int k = i - W1;
-        return k < 0 ? k + K : k;
-    }
-    return half - W2 + (i - n1);
-}
-
 __device__ __forceinline__ int d0(int k, int K) { return k <= (K >> 1) ? k : K - k; }
 __device__ __forceinline__ int dpi(int k, int K) {
     const int d = k - (K >> 1);
     return d < 0 ? -d : d;
-}
-
-// Slots of the union window per dimension.
-struct Slots {
-    int S[kMaxBins];
-    int W1[kMaxBins], W2[kMaxBins];
-};
-
-__device__ __forceinline__ Slots slots_of_grid(const GridD &g, const int *wmax) {
-    Slots s;
-#pragma unroll
-    for (int b = 0; b < kMaxBins; ++b) {
-        s.W1[b] = wmax[b];
-        s.W2[b] = wmax[kMaxBins + b];
-        s.S[b] = b < g.d ? slots_of(g.K[b], s.W1[b], s.W2[b]) : 1;
-    }
-    return s;
-}
-
-// Dimensions [0, nb) of the flattened slot index idx (last of them fastest)
-// -> k_b; returns the row-major grid index over those dimensions.
-__device__ __forceinline__ int64_t slot_ks(const GridD &g, const Slots &s, int nb, int64_t idx,
-                                           int (&k)[kMaxBins]) {
-    int64_t rem = idx;
-#pragma unroll
-    for (int b = kMaxBins - 1; b >= 0; --b) {
-        if (b >= nb) continue;
-        const int sb = (int)(rem % s.S[b]);
-        rem /= s.S[b];
-        k[b] = slot_k(sb, g.K[b], s.W1[b], s.W2[b]);
-    }
-    int64_t o = 0;
-#pragma unroll
-    for (int b = 0; b < kMaxBins; ++b)
-        if (b < nb) o = o * g.K[b] + k[b];
-    return o;
 }
 
 // One thread per slot of the union window (FP64 networks), one block row
@@ -342,17 +279,6 @@ constexpr int kSepTile = 32;     // slots per factor per CTA
 constexpr int kSepThreads = 256; // 16 x 16 threads, 2 x 2 points each
 constexpr int kSepRound = 16;    // trajectories per round
 
-// Per-trajectory constants of the factorised evaluation (one pass per chunk):
-// the bins' n_S in double-float and the exponent offsets.
-struct __align__(16) SepTraj {
-    df x[kMaxBins], y[kMaxBins];  // n_Sb
-    df m2, mp2;         // M_B, M'_B (offsets of the second factors)
-    df o1a, o1b;        // offsets of the first factors: +M_B, +M'_B + c2 + log inv
-    df rA;              // inv e^{c1} (<= 1)
-    int flags;          // 2: per-point FP64 route, 4: B term used, 8: rA == 1
-    int pad;
-};
-
 __global__ void k_sep_prep(const double *__restrict__ n_in, const double2 *__restrict__ nSd,
                            int64_t count, int d, SepTraj *__restrict__ out) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
@@ -390,8 +316,8 @@ __global__ void k_sep_prep(const double *__restrict__ n_in, const double2 *__res
         st.o1b = df_from_double(PB + c2 + linv);
         const double rA = exp(c1 + linv);
         st.rA = df_from_double(rA);
-        st.flags = (big ? 2 : 0) | (lwB >= -42.0 ? 4 : 0) | (rA == 1.0 ? 8 : 0);
-        st.pad = 0;
+        st.flags = (big ? kSepPoint : 0) | (lwB >= -42.0 ? kSepB : 0) | (rA == 1.0 ? kSepOne : 0);
+        st.top = (float)(lwB >= -42.0 ? fmax(MA + MB, lwB) : MA + MB);
         out[i] = st;
     }
 }
@@ -446,7 +372,8 @@ __global__ void __launch_bounds__(kSepThreads, 2)
     k_gf2d_df(const SepTraj *__restrict__ sep, const double *__restrict__ n_in,
               const double2 *__restrict__ nSd, const int *__restrict__ wmax, int64_t count,
               uint64_t e0, int n_sub, const GridD g, const double2 *__restrict__ tw,
-              const DfConsts K, double2 *__restrict__ acc, int64_t *__restrict__ counts) {
+              const DfConsts K, double2 *__restrict__ acc, int64_t *__restrict__ counts,
+              const int *__restrict__ rest, const SepMeta *__restrict__ meta, int rest_ld) {
     __shared__ float4 sA1[kSepRound][kSepTile], sB1[kSepRound][kSepTile];
     __shared__ float4 sA2[kSepRound][kSepTile], sB2[kSepRound][kSepTile];
     __shared__ SepTraj s_t[kSepRound];
@@ -461,8 +388,16 @@ __global__ void __launch_bounds__(kSepThreads, 2)
     const int tid = threadIdx.x;
     const int64_t first = (int64_t)(((uint64_t)r + (uint64_t)n_sub - e0 % (uint64_t)n_sub) %
                                     (uint64_t)n_sub);
-    const int64_t cnt_r = first < count ? (count - 1 - first) / n_sub + 1 : 0;
-    if (blockIdx.x == 0 && tid == 0) counts[r] += cnt_r;
+    int64_t cnt_r = first < count ? (count - 1 - first) / n_sub + 1 : 0;
+    // after the digit-product kernels: the sub-ensemble's list of what they left
+    if (rest) {
+        cnt_r = meta[r].g;
+        if (cnt_r == 0) return;
+        rest += (size_t)r * rest_ld;
+    } else if (blockIdx.x == 0 && tid == 0) {
+        counts[r] += cnt_r;
+    }
+    auto index = [&](int64_t q) { return rest ? (int64_t)rest[q] : first + q * n_sub; };
     const Slots sl = slots_of_grid(g, wmax);
     int64_t Sa = 1;
     for (int b = 0; b < d - 1; ++b) Sa *= sl.S[b];
@@ -534,8 +469,8 @@ __global__ void __launch_bounds__(kSepThreads, 2)
         const int nr = (int)((cnt_r - base) < kSepRound ? (cnt_r - base) : kSepRound);
         if (tid < kSepRound) {
             SepTraj st = {};
-            st.flags = 2 | 16;  // 16: no trajectory
-            if (tid < nr) st = sep[first + (base + tid) * n_sub];
+            st.flags = kSepPoint | kSepNone;
+            if (tid < nr) st = sep[index(base + tid)];
             s_t[tid] = st;
         }
         __syncthreads();
@@ -547,7 +482,7 @@ __global__ void __launch_bounds__(kSepThreads, 2)
             const int sidx = it % kSepTile;
             const SepTraj &st = s_t[j];
             float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A;
-            if (!(st.flags & 2) && s_ok[fac][sidx]) {
+            if (!(st.flags & kSepPoint) && s_ok[fac][sidx]) {
                 df l = {0.f, 0.f}, ph = {0.f, 0.f};
                 if (fac == 0) {
 #pragma unroll
@@ -574,7 +509,7 @@ __global__ void __launch_bounds__(kSepThreads, 2)
                     const df re = df_mul(e, cp), im = df_mul(e, sp);
                     A = make_float4(re.hi, im.hi, re.lo, im.lo);
                 }
-                if ((st.flags & 4) && eb.hi >= -87.0f) {
+                if ((st.flags & kSepB) && eb.hi >= -87.0f) {
                     const df e = df_exp_tab(eb, s_tab, K);
                     const df re = df_mul(e, cp), im = df_mul(e, sp);
                     B = make_float4(re.hi, -im.hi, re.lo, -im.lo);
@@ -600,9 +535,9 @@ __global__ void __launch_bounds__(kSepThreads, 2)
         __syncthreads();
         for (int j = 0; j < nr; ++j) {
             const int flags = s_t[j].flags;
-            if (flags & 2) {
+            if (flags & kSepPoint) {
                 // per-point FP64 route (huge phases or exponents)
-                const int64_t i = first + (base + j) * n_sub;
+                const int64_t i = index(base + j);
                 const double nn = n_in[i];
                 const double c1d = fmin(0.0, 2.0 * nn), c2d = -2.0 * fmax(nn, 0.0);
                 const double inv = 1.0 / (1.0 + exp(-2.0 * fabs(nn)));
@@ -647,8 +582,8 @@ __global__ void __launch_bounds__(kSepThreads, 2)
             // (< 2^-48 per term) is far below the double-float needs of the
             // large terms
             const float mA = s_mx[j][0][0] * s_mx[j][1][0];
-            const float mB = (flags & 4) ? s_mx[j][0][1] * s_mx[j][1][1] : 0.0f;
-            const bool rA1 = (flags & 8) != 0;
+            const float mB = (flags & kSepB) ? s_mx[j][0][1] * s_mx[j][1][1] : 0.0f;
+            const bool rA1 = (flags & kSepOne) != 0;
             if (mA >= 0x1p-63f && mA < 0x1p-25f) {
                 const float4 A1[2] = {sA1[j][2 * ty], sA1[j][2 * ty + 1]};
                 const float4 A2[2] = {sA2[j][2 * tx], sA2[j][2 * tx + 1]};
@@ -849,7 +784,22 @@ int launch_finalize2d(gbs_net *net, int64_t count) {
     return GBS_OK;
 }
 
-int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count) {
+// Work space of the digit-product kernels; ENOTSUP where the device has none to
+// spare (the outer-product kernel needs none).
+int reserve_gf2d_tc(gbs_net *net, int64_t KA, int KB, int64_t count) {
+    size_t bytes = 0;
+    gf2d_tc_piece(net->n_sub2, KA, KB, count, &bytes);
+    if (bytes <= net->gf2_bytes) return GBS_OK;
+    pool_free_raw(net->d_gf2, net->stream);
+    net->d_gf2 = nullptr;
+    net->gf2_bytes = 0;
+    if (pool_alloc(&net->d_gf2, bytes, net->stream, "joint generating functions")) return GBS_ENOTSUP;
+    net->gf2_bytes = bytes;
+    return GBS_OK;
+}
+
+int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count, int *launches) {
+    *launches = 0;
     if (count <= 0) return GBS_OK;
     const GridD g = grid_of(net);
     if (simt_precision(net->precision)) {
@@ -858,6 +808,7 @@ int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count) {
         k_gf2d<<<grid, kG2Threads, 0, net->stream>>>(net->d_n, net->d_nS2, net->d_win2,
                                                       net->d_wmax2, count, e0, net->n_sub2, g,
                                                       net->d_tw2, net->d_acc2, net->d_counts2);
+        *launches = 1;
     } else {
         static const DfConsts K = make_df_consts();
         // tiles of 32 x 32 slots over the whole grid; tiles past the chunk's
@@ -870,10 +821,33 @@ int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count) {
         k_sep_prep<<<blocks2(net, count), 256, 0, net->stream>>>(net->d_n, net->d_nS2, count,
                                                                  net->nbins, sep);
         GBS_LAUNCH_CHECK();
+        *launches = 1;
         auto kern = net->nbins == 2 ? k_gf2d_df<2> : net->nbins == 3 ? k_gf2d_df<3> : k_gf2d_df<4>;
+        int rc = GBS_ENOTSUP;
+        if (gf2d_tc_takes(net->n_sub2, KA, KB, count)) rc = reserve_gf2d_tc(net, KA, KB, count);
+        if (rc == GBS_OK) {
+            // pieces that fit in the work space
+            const int64_t piece = gf2d_tc_piece(net->n_sub2, KA, KB, count, nullptr);
+            for (int64_t p = 0; p < count; p += piece) {
+                const int64_t c = std::min(piece, count - p);
+                const int *rest;
+                const SepMeta *meta;
+                int ld;
+                if ((rc = launch_gf2d_tc(net, g, sep + p, c, e0 + (uint64_t)p, K, &rest, &meta, &ld)))
+                    return rc;
+                kern<<<g2, kSepThreads, 0, net->stream>>>(
+                    sep + p, net->d_n + p, net->d_nS2 + (size_t)net->nbins * p, net->d_wmax2, c,
+                    e0 + (uint64_t)p, net->n_sub2, g, net->d_tw2, K, net->d_acc2, net->d_counts2, rest,
+                    meta, ld);
+                GBS_LAUNCH_CHECK();
+                *launches += 4;
+            }
+            return GBS_OK;
+        }
         kern<<<g2, kSepThreads, 0, net->stream>>>(sep, net->d_n, net->d_nS2, net->d_wmax2, count,
                                                    e0, net->n_sub2, g, net->d_tw2, K, net->d_acc2,
-                                                   net->d_counts2);
+                                                   net->d_counts2, nullptr, nullptr, 0);
+        *launches += 1;
     }
     GBS_LAUNCH_CHECK();
     return GBS_OK;
