@@ -29,16 +29,24 @@ __host__ __device__ __forceinline__ int core_offset(int row, int k) {
     return (row >> 3) * 256 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
 }
 
-// v 2^s rounded to an integer (to nearest, halves away from zero), for
-// |v 2^s| <= 2^55 and a normal v; 0 below one half.
+// v 2^s rounded to an integer, to nearest and halves to even, for |v 2^s| <= 2^55 and
+// a normal v; 0 below one half.  (Two or three bits are dropped from a typical
+// amplitude, so a quarter of them are halves: rounding those away from zero
+// biased n_S by 0.7 2^-53.)
 __device__ __forceinline__ int64_t to_fixed(double v, int s) {
     const int64_t bits = __double_as_longlong(v);
     const int ex = (int)((bits >> 52) & 0x7ff) - 1075 + s;  // |v| 2^s = m 2^ex
     const int64_t m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
     int64_t x;
-    if (ex >= 0) x = m << ex;
-    else if (ex < -54) x = 0;
-    else x = ((m >> (-ex - 1)) + 1) >> 1;
+    if (ex >= 0) {
+        x = m << ex;
+    } else if (ex < -54) {
+        x = 0;
+    } else {
+        const int64_t t = m >> (-ex - 1);  // floor of twice the value
+        const bool up = (t << (-ex - 1)) != m || (t & 2);
+        x = (t + (up ? 1 : 0)) >> 1;
+    }
     return bits < 0 ? -x : x;
 }
 

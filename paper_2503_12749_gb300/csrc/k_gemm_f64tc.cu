@@ -28,10 +28,11 @@
 // for the FP64 FMA kernel (34 products at 0.84 of the measured BF16 rate; 6.27 with
 // a conversion for every sum and 32 columns read at once, f64tc_pipe.cuh);
 // N = M = 16, 16384 trajectories 0.049 against 0.150.  Root mean square error of
-// n_S against 113-bit arithmetic, relative to sum |alpha'_i| |beta'_i|:
-// N = 1000 1.9e-16 against 3.2e-16, N = 300 2.5e-16 against 3.1e-16, N = 64
-// 1.1e-16 against 1.3e-16, N = 16 3.1e-16 against 3.8e-16 (the input samples'
-// own rounding included in all).
+// n_S against 113-bit arithmetic, relative to sum |alpha'_i| |beta'_i|, real and
+// imaginary part (the input samples' own rounding included): N = 16 1.21e-16 and
+// 1.9e-17 against 1.18e-16 and 4.0e-17, N = 64 7.6e-17 and 1.2e-17 against 1.09e-16
+// and 3.8e-17, N = 200 8.7e-17 and 5.8e-18 against 1.17e-16 and 4.0e-17, N = 400
+// 8.8e-17 and 4.5e-18 against 1.12e-16 and 3.7e-17.
 //
 // Tile: 64 output modes (128 rows Re/Im) x 32 trajectories, as two sub-tiles
 // of 16 trajectories (16 alpha and 16 beta columns).  A sub-tile's eight D_d

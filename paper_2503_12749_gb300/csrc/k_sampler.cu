@@ -99,23 +99,28 @@ __global__ void __launch_bounds__(256)
         const int64_t i = i0 + lane;
         float *tile =
             B + (size_t)(i / kFp32TileSamples) * KB * kFp32BlockK * kRow + i % kFp32TileSamples;
-        double part = 0.0;
+        double p[4] = {0.0, 0.0, 0.0, 0.0};  // 32 chains of N / 32 terms, joined pairwise
         if (i < count)
             for (int j = warp; j < KB * kFp32BlockK; j += 8) {
                 double a = 0.0, b = 0.0;
                 if (j < N) {
                     amplitudes(sh, seed, e0 + (uint64_t)i, (uint32_t)j, sq[j], a, b);
-                    part = fma(a, b, part);
+                    const double s = fma(a, b, p[0]);
+                    p[0] = p[1];
+                    p[1] = p[2];
+                    p[2] = p[3];
+                    p[3] = s;
                 }
                 tile[(size_t)j * kRow] = (float)a;
                 tile[(size_t)j * kRow + kFp32TileSamples] = (float)b;
             }
-        s_n[warp][lane] = part;
+        s_n[warp][lane] = (p[0] + p[1]) + (p[2] + p[3]);
         __syncthreads();
         if (warp == 0 && i < count) {
+            double v[4];
 #pragma unroll
-            for (int w = 1; w < 8; ++w) part += s_n[w][lane];
-            n_out[i] = part;
+            for (int w = 0; w < 4; ++w) v[w] = s_n[2 * w][lane] + s_n[2 * w + 1][lane];
+            n_out[i] = (v[0] + v[1]) + (v[2] + v[3]);
         }
         __syncthreads();
     }
@@ -143,7 +148,7 @@ __global__ void __launch_bounds__(256, 2)
         const uint64_t e = e0 + (uint64_t)i;
         const int row = (int)(i & 15);
         uint8_t *tile = B + (size_t)(i / kTrajTile) * KB * kBStage + ((i >> 4) & 1) * kBSub;
-        double part = 0.0;
+        double sum[4] = {0.0, 0.0, 0.0, 0.0};  // chains of two modes of eight each
         if (i < count)
             for (int oct = (warp & (wpg - 1)) * 4 + (lane >> 3); oct < 2 * KB; oct += 4 * wpg) {
                 uint32_t da[kDigits][4], db[kDigits][4];
@@ -156,7 +161,7 @@ __global__ void __launch_bounds__(256, 2)
                         if (j < N) {
                             double a, b;
                             amplitudes(sh, seed, e, (uint32_t)j, sq[j], a, b);
-                            part = fma(a, b, part);
+                            sum[t >> 1] = fma(a, b, sum[t >> 1]);
                             const int s = 55 - col_exp[j];
                             xa[h] = to_fixed(a, s);
                             xb[h] = to_fixed(b, s);
@@ -180,13 +185,20 @@ __global__ void __launch_bounds__(256, 2)
                         make_uint4(db[q][0], db[q][1], db[q][2], db[q][3]);
                 }
             }
+        double part = (sum[0] + sum[1]) + (sum[2] + sum[3]);
         part += __shfl_xor_sync(0xffffffffu, part, 8);
         part += __shfl_xor_sync(0xffffffffu, part, 16);
         if (lane < 8) s_n[warp][lane] = part;
         __syncthreads();
+        // pairwise, as the shuffles: a chain of eight had 1.3 times its error
         if ((warp & (wpg - 1)) == 0 && lane < 8 && i < count) {
-            for (int w = 1; w < wpg; ++w) part += s_n[warp + w][lane];
-            n_out[i] = part;
+            if (wpg == 1) {
+                n_out[i] = part;
+            } else {
+                double v[4];
+                for (int w = 0; w < wpg / 2; ++w) v[w] = s_n[warp + 2 * w][lane] + s_n[warp + 2 * w + 1][lane];
+                n_out[i] = wpg == 2 ? v[0] : wpg == 4 ? v[0] + v[1] : (v[0] + v[1]) + (v[2] + v[3]);
+            }
         }
         __syncthreads();
     }
