@@ -75,15 +75,19 @@ __device__ __forceinline__ int64_t slot_ks(const GridD &g, const Slots &s, int n
 }
 
 // Per-trajectory constants of the factorised evaluation (one pass per chunk):
-// the bins' n_S in double-float and the exponent offsets.
-struct __align__(16) SepTraj {
-    df x[kMaxBins], y[kMaxBins];  // n_Sb
-    df m2, mp2;         // M_B, M'_B (offsets of the second factors)
-    df o1a, o1b;        // offsets of the first factors: +M_B, +M'_B + c2 + log inv
-    df rA;              // inv e^{c1} (<= 1)
+// the bins' n_S and the exponent offsets, V = df (BF16 networks) or double.
+template <typename V>
+struct __align__(16) SepTrajT {
+    V x[kMaxBins], y[kMaxBins];  // n_Sb
+    V m2, mp2;          // M_B, M'_B (offsets of the second factors)
+    V o1a, o1b;         // offsets of the first factors: +M_B, +M'_B + c2 + log inv
+    V rA;               // inv e^{c1} (<= 1)
     int flags;          // kSep... below
     float top;          // bound of the log of the first factor's magnitude
 };
+using SepTraj = SepTrajT<df>;
+using SepTraj64 = SepTrajT<double>;
+static_assert(sizeof(SepTraj) == sizeof(SepTraj64), "k_sep_lists reads flags and top of either");
 constexpr int kSepPoint = 2;   // per-point FP64 route
 constexpr int kSepB = 4;       // B term used
 constexpr int kSepOne = 8;     // rA == 1
@@ -92,6 +96,9 @@ constexpr int kSepNone = 16;   // no trajectory
 // their resolution is 2^-55 of the sub-ensemble's largest one, 2^-47 with this
 // bound, the double-float factors' own relative error
 constexpr float kSepTcTop = 5.5f;
+// the same for FP64 factors, whose exponents and phases, |n_Sb| of order 1 and more,
+// carry 2^-53 of themselves: below 2^3, rounded by at most 2^-53
+constexpr float kSepTcTop64 = 2.0f;
 
 // A sub-ensemble's lists of trajectories (k_sep_lists, for the digit-product
 // kernels): a = contracted A terms, x = B terms and (rA - 1) A terms
@@ -108,9 +115,10 @@ constexpr int kSepRest = 1 << 30;
 // whether they take `count` trajectories of this grid; a piece's bytes of work
 // space; one piece (list of the trajectories left over and their counts
 // returned for the outer-product kernel).
-bool gf2d_tc_takes(int n_sub, int64_t KA, int KB, int64_t count);
+bool gf2d_tc_takes(bool fp64, int n_sub, int64_t KA, int KB, int64_t count);
 int64_t gf2d_tc_piece(int n_sub, int64_t KA, int KB, int64_t count, size_t *bytes);
-int launch_gf2d_tc(gbs_net *net, const bin2d::GridD &g, const bin2d::SepTraj *sep, int64_t count,
+template <typename V>
+int launch_gf2d_tc(gbs_net *net, const bin2d::GridD &g, const bin2d::SepTrajT<V> *sep, int64_t count,
                    uint64_t e0, const DfConsts &K, const int **rest, const bin2d::SepMeta **meta,
                    int *rest_ld);
 

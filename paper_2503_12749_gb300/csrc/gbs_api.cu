@@ -440,11 +440,9 @@ int fix_estimator2d(gbs_net *net, int n_sub, const int *K) {
         (rc = net_alloc(net, &net->d_out2, (size_t)4 * grid, "out2")) ||
         (rc = net_alloc(net, &net->d_mo2, (size_t)kMaxBins, "window offsets")))
         return rc;
-    if (!simt_precision(net->precision)) {
-        if ((rc = pool_alloc(&net->d_sep2, (size_t)net->chunk * sep2_bytes_per_trajectory(),
-                             net->stream, "sep2")))
-            return rc;
-    }
+    if ((rc = pool_alloc(&net->d_sep2, (size_t)net->chunk * sep2_bytes_per_trajectory(), net->stream,
+                         "sep2")))
+        return rc;
     GBS_CUDA_TRY(cudaMemsetAsync(net->d_acc2, 0, accn * sizeof(double2), net->stream));
     GBS_CUDA_TRY(cudaMemsetAsync(net->d_counts2, 0, (size_t)n_sub * sizeof(int64_t), net->stream));
     if ((rc = launch_tables2d(net))) return rc;

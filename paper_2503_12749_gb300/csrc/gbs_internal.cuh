@@ -252,7 +252,7 @@ struct gbs_net {
     double2 *d_f2a = nullptr, *d_f2b = nullptr;  // [2][n_sub2][grid2] FFT work
     double *d_out2 = nullptr;       // [4][grid2]
     int64_t *d_mo2 = nullptr;       // [kMaxBins] DFT window offsets
-    void *d_sep2 = nullptr;         // [chunk] per-trajectory constants (BF16 networks)
+    void *d_sep2 = nullptr;         // [chunk] per-trajectory constants
     void *d_gf2 = nullptr;          // work space of the digit-product kernels (k_gf2d_tc.cu)
     size_t gf2_bytes = 0;
 };

@@ -146,14 +146,15 @@ __device__ __forceinline__ int dpi(int k, int K) {
     return d < 0 ? -d : d;
 }
 
-// One thread per slot of the union window (FP64 networks), one block row
-// per sub-ensemble r; each thread adds its sub-ensemble's trajectories in
-// increasing order.
+// One thread per slot of the union window (FP64 and FP32 networks), one block row
+// per sub-ensemble r; each thread adds its sub-ensemble's trajectories (or those
+// that the digit contraction left) in increasing order.
 __global__ void __launch_bounds__(kG2Threads)
     k_gf2d(const double *__restrict__ n_in, const double2 *__restrict__ nSd,
            const WindowD *__restrict__ win_in, const int *__restrict__ wmax, int64_t count,
            uint64_t e0, int n_sub, const GridD g, const double2 *__restrict__ tw,
-           double2 *__restrict__ acc, int64_t *__restrict__ counts) {
+           double2 *__restrict__ acc, int64_t *__restrict__ counts, const int *__restrict__ rest,
+           const SepMeta *__restrict__ meta, int rest_ld) {
     __shared__ double s_x[kG2Tile][kMaxBins], s_y[kG2Tile][kMaxBins];
     __shared__ double s_c1[kG2Tile], s_c2[kG2Tile], s_inv[kG2Tile];
     __shared__ WindowD s_w[kG2Tile];
@@ -165,8 +166,15 @@ __global__ void __launch_bounds__(kG2Threads)
     const int64_t slot = (int64_t)blockIdx.x * kG2Threads + threadIdx.x;
     const int64_t first = (int64_t)(((uint64_t)r + (uint64_t)n_sub - e0 % (uint64_t)n_sub) %
                                     (uint64_t)n_sub);
-    const int64_t cnt_r = first < count ? (count - 1 - first) / n_sub + 1 : 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) counts[r] += cnt_r;
+    int64_t cnt_r = first < count ? (count - 1 - first) / n_sub + 1 : 0;
+    // after the digit-product kernels: the sub-ensemble's list of what they left
+    if (rest) {
+        cnt_r = meta[r].g;
+        if (cnt_r == 0) return;
+        rest += (size_t)r * rest_ld;
+    } else if (blockIdx.x == 0 && threadIdx.x == 0) {
+        counts[r] += cnt_r;
+    }
     if ((int64_t)blockIdx.x * kG2Threads >= total) return;  // block past the grid
     const bool valid = slot < total;
     int k[kMaxBins] = {0, 0, 0, 0}, a0[kMaxBins], api[kMaxBins];
@@ -183,7 +191,7 @@ __global__ void __launch_bounds__(kG2Threads)
     for (int64_t base = 0; base < cnt_r; base += kG2Tile) {
         const int64_t q = base + threadIdx.x;
         if (q < cnt_r) {
-            const int64_t i = first + q * n_sub;
+            const int64_t i = rest ? (int64_t)rest[q] : first + q * n_sub;
             const double nn = n_in[i];
 #pragma unroll
             for (int b = 0; b < kMaxBins; ++b) {
@@ -279,19 +287,23 @@ constexpr int kSepTile = 32;     // slots per factor per CTA
 constexpr int kSepThreads = 256; // 16 x 16 threads, 2 x 2 points each
 constexpr int kSepRound = 16;    // trajectories per round
 
+__device__ __forceinline__ void put(df &o, double v) { o = df_from_double(v); }
+__device__ __forceinline__ void put(double &o, double v) { o = v; }
+
+template <typename V>
 __global__ void k_sep_prep(const double *__restrict__ n_in, const double2 *__restrict__ nSd,
-                           int64_t count, int d, SepTraj *__restrict__ out) {
+                           int64_t count, int d, SepTrajT<V> *__restrict__ out) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
         const double nn = n_in[i];
-        SepTraj st;
+        SepTrajT<V> st;
         double MA = 0.0, PA = 0.0, phA = 0.0, MB = 0.0, PB = 0.0, phB = 0.0;
         bool bad = false;
 #pragma unroll
         for (int b = 0; b < kMaxBins; ++b) {
             const double2 v = b < d ? nSd[(size_t)d * i + b] : make_double2(0.0, 0.0);
-            st.x[b] = df_from_double(v.x);
-            st.y[b] = df_from_double(v.y);
+            put(st.x[b], v.x);
+            put(st.y[b], v.y);
             if (b >= d) continue;
             const double m1 = max_term1(v.x, v.y), m2 = max_term2(v.x, v.y);
             const double ph = fabs(v.x) + 2.0 * fabs(v.y);
@@ -310,12 +322,12 @@ __global__ void k_sep_prep(const double *__restrict__ n_in, const double2 *__res
         const double linv = -log1p(exp(-2.0 * fabs(nn)));
         const double lwB = PA + PB + c2 + linv;
         const bool big = bad || phA >= 6000.0 || phB >= 6000.0 || MA + MB > 40.0 || lwB > 40.0;
-        st.m2 = df_from_double(MB);
-        st.mp2 = df_from_double(PB);
-        st.o1a = df_from_double(MB);
-        st.o1b = df_from_double(PB + c2 + linv);
+        put(st.m2, MB);
+        put(st.mp2, PB);
+        put(st.o1a, MB);
+        put(st.o1b, PB + c2 + linv);
         const double rA = exp(c1 + linv);
-        st.rA = df_from_double(rA);
+        put(st.rA, rA);
         st.flags = (big ? kSepPoint : 0) | (lwB >= -42.0 ? kSepB : 0) | (rA == 1.0 ? kSepOne : 0);
         st.top = (float)(lwB >= -42.0 ? fmax(MA + MB, lwB) : MA + MB);
         out[i] = st;
@@ -802,54 +814,59 @@ int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count, int *launches) {
     *launches = 0;
     if (count <= 0) return GBS_OK;
     const GridD g = grid_of(net);
-    if (simt_precision(net->precision)) {
-        // blocks for the whole grid; blocks past the chunk's union window return
-        dim3 grid((unsigned)((net->grid2 + kG2Threads - 1) / kG2Threads), (unsigned)net->n_sub2);
-        k_gf2d<<<grid, kG2Threads, 0, net->stream>>>(net->d_n, net->d_nS2, net->d_win2,
-                                                      net->d_wmax2, count, e0, net->n_sub2, g,
-                                                      net->d_tw2, net->d_acc2, net->d_counts2);
-        *launches = 1;
-    } else {
-        static const DfConsts K = make_df_consts();
-        // tiles of 32 x 32 slots over the whole grid; tiles past the chunk's
-        // union window return at once
-        const int KB = net->Kd[net->nbins - 1];
-        const int64_t KA = net->grid2 / KB;
-        const int64_t tiles = ((KA + kSepTile - 1) / kSepTile) * ((KB + kSepTile - 1) / kSepTile);
-        dim3 g2((unsigned)tiles, (unsigned)net->n_sub2);
-        SepTraj *sep = static_cast<SepTraj *>(net->d_sep2);
-        k_sep_prep<<<blocks2(net, count), 256, 0, net->stream>>>(net->d_n, net->d_nS2, count,
-                                                                 net->nbins, sep);
+    static const DfConsts K = make_df_consts();
+    const bool simt = simt_precision(net->precision);
+    const int KB = net->Kd[net->nbins - 1];
+    const int64_t KA = net->grid2 / KB;
+    int rc = GBS_ENOTSUP;
+    if (gf2d_tc_takes(simt, net->n_sub2, KA, KB, count)) rc = reserve_gf2d_tc(net, KA, KB, count);
+    const bool tc = rc == GBS_OK;
+    SepTraj *sep = static_cast<SepTraj *>(net->d_sep2);
+    SepTraj64 *sep64 = static_cast<SepTraj64 *>(net->d_sep2);
+    if (tc || !simt) {
+        if (simt)
+            k_sep_prep<double><<<blocks2(net, count), 256, 0, net->stream>>>(
+                net->d_n, net->d_nS2, count, net->nbins, sep64);
+        else
+            k_sep_prep<df><<<blocks2(net, count), 256, 0, net->stream>>>(net->d_n, net->d_nS2, count,
+                                                                         net->nbins, sep);
         GBS_LAUNCH_CHECK();
-        *launches = 1;
-        auto kern = net->nbins == 2 ? k_gf2d_df<2> : net->nbins == 3 ? k_gf2d_df<3> : k_gf2d_df<4>;
-        int rc = GBS_ENOTSUP;
-        if (gf2d_tc_takes(net->n_sub2, KA, KB, count)) rc = reserve_gf2d_tc(net, KA, KB, count);
-        if (rc == GBS_OK) {
-            // pieces that fit in the work space
-            const int64_t piece = gf2d_tc_piece(net->n_sub2, KA, KB, count, nullptr);
-            for (int64_t p = 0; p < count; p += piece) {
-                const int64_t c = std::min(piece, count - p);
-                const int *rest;
-                const SepMeta *meta;
-                int ld;
-                if ((rc = launch_gf2d_tc(net, g, sep + p, c, e0 + (uint64_t)p, K, &rest, &meta, &ld)))
-                    return rc;
-                kern<<<g2, kSepThreads, 0, net->stream>>>(
-                    sep + p, net->d_n + p, net->d_nS2 + (size_t)net->nbins * p, net->d_wmax2, c,
-                    e0 + (uint64_t)p, net->n_sub2, g, net->d_tw2, K, net->d_acc2, net->d_counts2, rest,
-                    meta, ld);
-                GBS_LAUNCH_CHECK();
-                *launches += 4;
-            }
-            return GBS_OK;
-        }
-        kern<<<g2, kSepThreads, 0, net->stream>>>(sep, net->d_n, net->d_nS2, net->d_wmax2, count,
-                                                   e0, net->n_sub2, g, net->d_tw2, K, net->d_acc2,
-                                                   net->d_counts2, nullptr, nullptr, 0);
         *launches += 1;
     }
-    GBS_LAUNCH_CHECK();
+    // with the digit contraction: pieces that fit in its work space
+    const int64_t piece = tc ? gf2d_tc_piece(net->n_sub2, KA, KB, count, nullptr) : count;
+    for (int64_t p = 0; p < count; p += piece) {
+        const int64_t c = std::min(piece, count - p);
+        const uint64_t e = e0 + (uint64_t)p;
+        const int *rest = nullptr;
+        const SepMeta *meta = nullptr;
+        int ld = 0;
+        if (tc) {
+            rc = simt ? launch_gf2d_tc(net, g, sep64 + p, c, e, K, &rest, &meta, &ld)
+                      : launch_gf2d_tc(net, g, sep + p, c, e, K, &rest, &meta, &ld);
+            if (rc) return rc;
+            *launches += 3;
+        }
+        const double *n = net->d_n + p;
+        const double2 *nSd = net->d_nS2 + (size_t)net->nbins * p;
+        if (simt) {
+            // blocks for the whole grid; blocks past the chunk's union window return
+            dim3 grid((unsigned)((net->grid2 + kG2Threads - 1) / kG2Threads), (unsigned)net->n_sub2);
+            k_gf2d<<<grid, kG2Threads, 0, net->stream>>>(n, nSd, net->d_win2 + p, net->d_wmax2, c, e,
+                                                          net->n_sub2, g, net->d_tw2, net->d_acc2,
+                                                          net->d_counts2, rest, meta, ld);
+        } else {
+            // tiles of 32 x 32 slots over the whole grid, likewise
+            const int64_t tiles = ((KA + kSepTile - 1) / kSepTile) * ((KB + kSepTile - 1) / kSepTile);
+            dim3 grid((unsigned)tiles, (unsigned)net->n_sub2);
+            auto kern = net->nbins == 2 ? k_gf2d_df<2> : net->nbins == 3 ? k_gf2d_df<3> : k_gf2d_df<4>;
+            kern<<<grid, kSepThreads, 0, net->stream>>>(sep + p, n, nSd, net->d_wmax2, c, e, net->n_sub2,
+                                                        g, net->d_tw2, K, net->d_acc2, net->d_counts2,
+                                                        rest, meta, ld);
+        }
+        GBS_LAUNCH_CHECK();
+        *launches += 1;
+    }
     return GBS_OK;
 }
 

@@ -1,12 +1,13 @@
 // The joint generating functions of d = 2..4 output bins as exact integer
-// contractions on the tensor cores (BF16 networks).
+// contractions on the tensor cores.
 //
 // With the factorisation of k_bin2d.cu a sub-ensemble's sums are contractions
 // over its trajectories,
 //   sum G_+P = sum_e A_1 A_2,   sum G_mP = sum G_+P + sum_e [B_1 B_2 + (rA - 1) A_1 A_2],
 // of complex vectors on the first bins' flattened slots and the last bin's.
-// The factors are evaluated once per (trajectory, slot) in double-float (the
-// outer-product kernel evaluates them once per tile of 32 x 32 slots), written
+// The factors are evaluated once per (trajectory, slot) in double-float (BF16
+// networks; the outer-product kernel evaluates them once per tile of 32 x 32
+// slots) or FP64 (the others; k_gf2d evaluates every grid point), written
 // as 56-bit fixed-point numbers of seven balanced 8-bit digits, and the digit
 // products are contracted without rounding by the pipeline of the FP64 GEMM
 // (f64tc_pipe.cuh): rows are (slot of the first factor, Re / Im), columns the
@@ -14,9 +15,10 @@
 //   Re row: (A_1r, -A_1i), Im row: (A_1i, A_1r) against (A_2r, A_2i).
 // The second factors are at most 1, the first ones of a sub-ensemble below 2^f
 // of their largest: resolutions 2^-56 and 2^(f - 56), against 2^-46 relative of
-// the double-float factors.  Trajectories whose first factor may exceed
-// e^kSepTcTop, or whose phase or exponent is beyond the double-float functions,
-// are listed for the outer-product kernel.  The integer sums do not depend on
+// the double-float factors (FP64 ones have f <= 3, 2^-53 of exponents and phases, and
+// sums that were rounded at every term).  Trajectories whose first factor may exceed e^kSepTcTop
+// (e^kSepTcTop64), or whose phase or exponent is beyond the double-float functions,
+// are listed for the general kernels (k_gf2d_df, k_gf2d).  The integer sums do not depend on
 // their order, so the lists are compacted.
 //
 // Why: the double-float outer products are 2 x 16 packed FP32 instructions per
@@ -28,8 +30,10 @@
 // and the drain of the sums is not fully covered, f64tc_pipe.cuh).
 #include "bin2d.cuh"
 #include "f64tc_pipe.cuh"
+#include "gf64.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace gbs {
 namespace {
@@ -53,8 +57,9 @@ constexpr size_t kWorkBytes = (size_t)2 << 30;
 // of a tile's columns are padding).  Whole gbs_sample_nd calls, outer products ->
 // contraction (us): 100 sub-ensembles on 64 x 64 of 16 trajectories 151 -> 164, 32
 // 158 -> 157, 64 271 -> 220; 128 x 128 of 32 324 -> 256, 512 2913 -> 1038; 32 x 32 of
-// 32 139 -> 164, 10 of 2000 2463 -> 848; 50 of 1000 on 32 x 32 x 32 9658 -> 5641.
-constexpr int64_t kMinPerSub = 32, kMinPerSub32 = 128;
+// 32 139 -> 164, 10 of 2000 2463 -> 848; 50 of 1000 on 32 x 32 x 32 9658 -> 5641.  FP64
+// networks, whose general kernel is ten times slower: 100 of 8 on 32 x 32 342 -> 226.
+constexpr int64_t kMinPerSub = 32, kMinPerSub32 = 128, kMinPerSub64 = 8;
 
 // Offsets of the work space for `q` (a multiple of 8) trajectories per
 // sub-ensemble: K blocks r cap + [0, q / 8) hold the A terms, the next 2 q / 8
@@ -77,9 +82,10 @@ struct Work {
 };
 
 // One block per sub-ensemble: its lists [A: q][X: 2 q][rest: q], in order.
+template <typename V>
 __global__ void __launch_bounds__(kListThreads)
-    k_sep_lists(const SepTraj *__restrict__ sep, int64_t count, uint64_t e0, int n_sub, int q,
-                int *__restrict__ lists, SepMeta *__restrict__ meta, int64_t *__restrict__ counts) {
+    k_sep_lists(const SepTrajT<V> *__restrict__ sep, float most, int64_t count, uint64_t e0, int n_sub,
+                int q, int *__restrict__ lists, SepMeta *__restrict__ meta, int64_t *__restrict__ counts) {
     __shared__ int s_sum[kListThreads / 32];
     __shared__ unsigned s_top[kListThreads / 32];
     const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -97,7 +103,7 @@ __global__ void __launch_bounds__(kListThreads)
         if (t < cnt_r) {
             flags = sep[i].flags;
             const float b = sep[i].top;
-            in = !(flags & kSepPoint) && b <= kSepTcTop;
+            in = !(flags & kSepPoint) && b <= most;
             left = !in;
             if (in) top = fmaxf(top, b);
         }
@@ -147,6 +153,32 @@ __device__ __forceinline__ int64_t df_fixed(float hi, float lo, float scale) {
     const int top = __float2int_rn(h);
     const float rest = (h - (float)top) * 0x1p32f;  // exact, |.| <= 2^31
     return ((int64_t)top << 32) + __float2int_rn(rest) + __float2int_rn(lo * scale * 0x1p32f);
+}
+
+// v 2^s rounded to an integer, |v 2^s| <= 2^55 (to_fixed takes normal numbers).
+__device__ __forceinline__ int64_t to_fixed_any(double v, int s) {
+    return fabs(v) < 0x1p-60 ? 0 : to_fixed(v, s);
+}
+
+// Digits (re, im) of four trajectories of slot `slot` (0..63) of a tile: rows
+// (re, -im) and (im, re), or a column (re, im); `half` of the K block.
+__device__ __forceinline__ void store_row(uint8_t *tile, int slot, int half, const uint32_t (&w)[kDigits][4]) {
+    uint8_t *o = tile + core_offset(2 * slot, 8 * half);
+    constexpr uint32_t neg = 0x80000000u;
+#pragma unroll
+    for (int p = 0; p < kDigits; ++p) {
+        *reinterpret_cast<uint4 *>(o + p * kASlice) =
+            make_uint4(w[p][0] ^ neg, w[p][1] ^ neg, w[p][2] ^ neg, w[p][3] ^ neg);
+        *reinterpret_cast<uint4 *>(o + p * kASlice + 16) =
+            make_uint4(__byte_perm(w[p][0], 0u, 0x1032), __byte_perm(w[p][1], 0u, 0x1032),
+                       __byte_perm(w[p][2], 0u, 0x1032), __byte_perm(w[p][3], 0u, 0x1032));
+    }
+}
+__device__ __forceinline__ void store_col(uint8_t *tile, int slot, int half, const uint32_t (&w)[kDigits][4]) {
+    uint8_t *o = tile + (slot >> 5) * kBSub + core_offset(slot & 31, 8 * half);
+#pragma unroll
+    for (int p = 0; p < kDigits; ++p)
+        *reinterpret_cast<uint4 *>(o + p * kBSlice) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
 }
 
 // The operands' digits: a thread holds one slot of either factor and takes four
@@ -200,11 +232,9 @@ __global__ void __launch_bounds__(kDigThreads, 3)
                 sn[b] = df_from_double(t.y);
             }
         }
-        // first factors below 2^f, second factors at most 1 (2^54: room for
-        // their rounding); df_fixed multiplies by 2^32
-        const float scale = __uint_as_float((uint32_t)(127 - 32 + (row ? 55 - mr.f : 54)) << 23);
-        const uint32_t off = row ? (uint32_t)core_offset(2 * (slot & 63), 0)
-                                 : (uint32_t)(((slot >> 5) & 1) * kBSub + core_offset(slot & 31, 0));
+        // first factors below 2^f, second factors at most 1; df_fixed multiplies
+        // by 2^32
+        const float scale = __uint_as_float((uint32_t)(127 - 32 + 55 - (row ? mr.f : 0)) << 23);
         for (int u0 = blockIdx.x * kQuads; u0 < qa + qx; u0 += gridDim.x * kQuads) {
             __syncthreads();
             for (int j = tid; j < 4 * kQuads * kTrajWords; j += kDigThreads) {
@@ -277,27 +307,97 @@ __global__ void __launch_bounds__(kDigThreads, 3)
                     for (int p = 0; p < kDigits; ++p) w[p][t + 1] = dg[p];
                 }
                 const size_t kb = (isx ? kb_x : kb_a) + (quad >> 1);
-                const uint32_t half = (quad & 1) * 128;
-                if (row) {
-                    uint8_t *o = imgA + (kb * mt + (slot >> 6)) * kAStage + off + half;
-#pragma unroll
-                    for (int p = 0; p < kDigits; ++p) {
-                        // Re row (re, -im), Im row (im, re)
-                        constexpr uint32_t neg = 0x80000000u;
-                        *reinterpret_cast<uint4 *>(o + p * kASlice) =
-                            make_uint4(w[p][0] ^ neg, w[p][1] ^ neg, w[p][2] ^ neg, w[p][3] ^ neg);
-                        *reinterpret_cast<uint4 *>(o + p * kASlice + 16) =
-                            make_uint4(__byte_perm(w[p][0], 0u, 0x1032), __byte_perm(w[p][1], 0u, 0x1032),
-                                       __byte_perm(w[p][2], 0u, 0x1032), __byte_perm(w[p][3], 0u, 0x1032));
-                    }
-                } else {
-                    uint8_t *o = imgB + (kb * ct + (slot >> 6)) * kBStage + off + half;
-#pragma unroll
-                    for (int p = 0; p < kDigits; ++p)
-                        *reinterpret_cast<uint4 *>(o + p * kBSlice) =
-                            make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
-                }
+                if (row) store_row(imgA + (kb * mt + (slot >> 6)) * kAStage, slot & 63, quad & 1, w);
+                else store_col(imgB + (kb * ct + (slot >> 6)) * kBStage, slot & 63, quad & 1, w);
             }
+        }
+    }
+}
+
+// The same from FP64 factors (FP64 and FP32 networks): bound by the FP64 pipe's
+// exponentials, sines and cosines.
+template <int D>
+__global__ void __launch_bounds__(kDigThreads)
+    k_sep_digits64(const SepTraj64 *__restrict__ sep, const SepMeta *__restrict__ meta,
+                   const int *__restrict__ lists, int q, const int *__restrict__ wmax, const GridD g,
+                   const double2 *__restrict__ tw, const Gf64Tables tabs,
+                   uint8_t *__restrict__ imgA, uint8_t *__restrict__ imgB) {
+    __shared__ Gf64Tables s_tab;
+    constexpr int d = D;
+    const int tid = threadIdx.x, r = blockIdx.y;
+    if (tid < 64) s_tab.exp2[tid] = tabs.exp2[tid];
+    for (int t = tid; t < 256; t += kDigThreads) {
+        s_tab.sn[t] = tabs.sn[t];
+        s_tab.cs[t] = tabs.cs[t];
+    }
+    __syncthreads();
+    const Slots sl = slots_of_grid(g, wmax);
+    int Sa = 1;
+    for (int b = 0; b < d - 1; ++b) Sa *= sl.S[b];
+    const int Sb = sl.S[d - 1];
+    const int mt = (Sa + kSlotTile - 1) / kSlotTile, ct = (Sb + kSlotTile - 1) / kSlotTile;
+    const int Ra = (Sa + 31) / 32 * 32;
+    const SepMeta mr = meta[r];
+    const int qa = 2 * ((mr.a + kEntryBlock - 1) / kEntryBlock);
+    const int qx = 2 * ((mr.x + kEntryBlock - 1) / kEntryBlock);
+    const int *la = lists + (size_t)r * 4 * q;
+    const size_t kb_a = (size_t)r * 3 * (q / kEntryBlock), kb_x = kb_a + q / kEntryBlock;
+    for (int s = tid; s < Ra + Sb; s += kDigThreads) {
+        const bool row = s < Ra;
+        const int slot = row ? s : s - Ra;
+        if (row && slot >= Sa) continue;
+        double cm[d - 1], sn[d - 1];
+        {
+            int k[kMaxBins] = {0, 0, 0, 0};
+            if (row) slot_ks(g, sl, d - 1, slot, k);
+            else k[0] = slot_k(slot, g.K[d - 1], sl.W1[d - 1], sl.W2[d - 1]);
+#pragma unroll
+            for (int b = 0; b < d - 1; ++b) {
+                const double2 t = tw[row ? g.Koff[b] + k[b] : g.Koff[d - 1] + k[0]];
+                cm[b] = t.x;
+                sn[b] = t.y;
+            }
+        }
+        const int shift = 55 - (row ? mr.f : 0);
+        for (int u = blockIdx.x; u < qa + qx; u += gridDim.x) {
+            const bool isx = u >= qa;
+            const int quad = isx ? u - qa : u;
+            const int *list = (isx ? la + q : la) + 4 * quad;
+            const int left = (isx ? mr.x : mr.a) - 4 * quad;
+            uint32_t w[kDigits][4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                int64_t xr = 0, xi = 0;
+                if (t < left) {
+                    const int entry = list[t];
+                    const SepTraj64 &st = sep[entry & (kSepRest - 1)];
+                    const bool rest = (entry & kSepRest) != 0, isb = isx && !rest;
+                    double l = 0.0, ph = 0.0;
+                    if (row) {
+#pragma unroll
+                        for (int b = 0; b < d - 1; ++b) {
+                            l += cm[b] * st.x[b] - sn[b] * st.y[b];
+                            ph += sn[b] * st.x[b] + cm[b] * st.y[b];
+                        }
+                    } else {
+                        l = cm[0] * st.x[d - 1] - sn[0] * st.y[d - 1];
+                        ph = sn[0] * st.x[d - 1] + cm[0] * st.y[d - 1];
+                    }
+                    const double ofs = row ? (isb ? st.o1b : st.o1a) : -(isb ? st.mp2 : st.m2);
+                    double si, co, e = exp_tab64((isb ? -l : l) + ofs, s_tab);
+                    sincos_tab64(ph, s_tab, si, co);
+                    if (row && rest) e *= st.rA - 1.0;
+                    xr = to_fixed_any(e * co, shift);
+                    xi = to_fixed_any(e * (isb ? -si : si), shift);
+                }
+                uint32_t dg[kDigits];
+                digit_pairs(xr, xi, dg);
+#pragma unroll
+                for (int p = 0; p < kDigits; ++p) w[p][t] = dg[p];
+            }
+            const size_t kb = (isx ? kb_x : kb_a) + (quad >> 1);
+            if (row) store_row(imgA + (kb * mt + (slot >> 6)) * kAStage, slot & 63, quad & 1, w);
+            else store_col(imgB + (kb * ct + (slot >> 6)) * kBStage, slot & 63, quad & 1, w);
         }
     }
 }
@@ -364,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int b = 0; b < g.d; ++b) grid *= g.K[b];
                 int k[kMaxBins] = {0, 0, 0, 0};
                 const int64_t oA = slot_ks(g, sl, g.d - 1, slot, k);
-                const int f = meta[r].f + 1 - 70;
+                const int f = meta[r].f - 70;
                 double *o = acc + 2 * ((size_t)(part ? r : n_sub + r) * grid + (size_t)oA * KB) + (row & 1);
                 // (one addition per element and launch: the sums stay reproducible;
                 // reductions at L2, since a load, an addition and a store each wait
@@ -382,9 +482,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 }  // namespace
 
 // (rows, 128 a tile, are 64 slots of the first factor)
-bool gf2d_tc_takes(int n_sub, int64_t KA, int KB, int64_t count) {
+bool gf2d_tc_takes(bool fp64, int n_sub, int64_t KA, int KB, int64_t count) {
     if (KA < 32 || KB < 32 || KA > (1 << 20)) return false;
-    if (count / n_sub < (KB > 32 ? kMinPerSub : kMinPerSub32)) return false;
+    if (count / n_sub < (fp64 ? kMinPerSub64 : KB > 32 ? kMinPerSub : kMinPerSub32)) return false;
     return Work(n_sub, KA, KB, kMinPerSub).bytes <= kWorkBytes;
 }
 
@@ -398,7 +498,8 @@ int64_t gf2d_tc_piece(int n_sub, int64_t KA, int KB, int64_t count, size_t *byte
     return piece;
 }
 
-int launch_gf2d_tc(gbs_net *net, const GridD &g, const SepTraj *sep, int64_t count, uint64_t e0,
+template <typename V>
+int launch_gf2d_tc(gbs_net *net, const GridD &g, const SepTrajT<V> *sep, int64_t count, uint64_t e0,
                    const DfConsts &K, const int **rest, const SepMeta **meta, int *rest_ld) {
     const int n_sub = net->n_sub2, KB = g.K[g.d - 1];
     const int64_t KA = net->grid2 / KB;
@@ -407,15 +508,24 @@ int launch_gf2d_tc(gbs_net *net, const GridD &g, const SepTraj *sep, int64_t cou
     uint8_t *base = static_cast<uint8_t *>(net->d_gf2);
     int *lists = reinterpret_cast<int *>(base + w.lists);
     SepMeta *m = reinterpret_cast<SepMeta *>(base + w.meta);
-    k_sep_lists<<<n_sub, kListThreads, 0, net->stream>>>(sep, count, e0, n_sub, w.q, lists, m,
-                                                         net->d_counts2);
+    constexpr bool fp64 = std::is_same<V, double>::value;
+    k_sep_lists<<<n_sub, kListThreads, 0, net->stream>>>(sep, fp64 ? kSepTcTop64 : kSepTcTop, count, e0,
+                                                         n_sub, w.q, lists, m, net->d_counts2);
     GBS_LAUNCH_CHECK();
     // about five blocks per block slot of the chip
     const int groups = (2 * w.cap + kQuads - 1) / kQuads;
     const int per = std::max(1, std::min(groups, 16 * net->sm_count / n_sub));
-    auto digits = g.d == 2 ? k_sep_digits<2> : g.d == 3 ? k_sep_digits<3> : k_sep_digits<4>;
-    digits<<<dim3((unsigned)per, (unsigned)n_sub), kDigThreads, 0, net->stream>>>(
-        sep, m, lists, w.q, net->d_wmax2, g, net->d_tw2, K, base, base + w.img_b);
+    const dim3 grid((unsigned)per, (unsigned)n_sub);
+    if constexpr (fp64) {
+        static const Gf64Tables T = make_gf64_tables();
+        auto digits = g.d == 2 ? k_sep_digits64<2> : g.d == 3 ? k_sep_digits64<3> : k_sep_digits64<4>;
+        digits<<<grid, kDigThreads, 0, net->stream>>>(sep, m, lists, w.q, net->d_wmax2, g, net->d_tw2,
+                                                      T, base, base + w.img_b);
+    } else {
+        auto digits = g.d == 2 ? k_sep_digits<2> : g.d == 3 ? k_sep_digits<3> : k_sep_digits<4>;
+        digits<<<grid, kDigThreads, 0, net->stream>>>(sep, m, lists, w.q, net->d_wmax2, g, net->d_tw2, K,
+                                                      base, base + w.img_b);
+    }
     GBS_LAUNCH_CHECK();
     GBS_CUDA_TRY(cudaFuncSetAttribute(k_gf2d_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kPipeBytes));
     const int64_t tiles = (int64_t)n_sub * ((KA + kSlotTile - 1) / kSlotTile) *
@@ -429,5 +539,10 @@ int launch_gf2d_tc(gbs_net *net, const GridD &g, const SepTraj *sep, int64_t cou
     *rest_ld = 4 * w.q;
     return GBS_OK;
 }
+
+template int launch_gf2d_tc(gbs_net *, const GridD &, const SepTrajT<df> *, int64_t, uint64_t,
+                            const DfConsts &, const int **, const SepMeta **, int *);
+template int launch_gf2d_tc(gbs_net *, const GridD &, const SepTrajT<double> *, int64_t, uint64_t,
+                            const DfConsts &, const int **, const SepMeta **, int *);
 
 }  // namespace gbs
