@@ -170,7 +170,8 @@ int gbs_sample_nd(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E
  * m_b = m_offset[b] .. m_offset[b] + K_b - 1, P = mean_r Re P_r, sigma =
  * std_r / sqrt(N_R).  m_offset: host, d values.  Host outputs of prod K_b
  * doubles each, row-major over (m_1, .., m_d); any may be NULL.
- * Synchronises the stream.  Errors: EINVAL, ECUDA.
+ * Synchronises the stream.  Errors: EINVAL, ECUDA, ETIMEOUT (a kernel gave up
+ * waiting on its pipeline: the sums are not meaningful; gbs_reset).
  */
 int gbs_binned_counts_nd(gbs_net_t net, const int64_t *m_offset, double *P_mP, double *sig_mP,
                          double *P_plusP, double *sig_plusP);
@@ -200,7 +201,7 @@ int gbs_sample_2d(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E
  * m_b = m_b_offset .. m_b_offset + K_b - 1, P = mean_r Re P_r, sigma =
  * std_r / sqrt(N_R).  Host outputs of K1*K2 doubles each, [m_1][m_2]
  * row-major; any may be NULL.  Synchronises the stream.  Errors: EINVAL,
- * ECUDA.
+ * ECUDA, ETIMEOUT.
  */
 int gbs_binned_counts_2d(gbs_net_t net, int64_t m1_offset, int64_t m2_offset, double *P_mP,
                          double *sig_mP, double *P_plusP, double *sig_plusP);

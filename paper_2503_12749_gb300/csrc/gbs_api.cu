@@ -1275,7 +1275,14 @@ int gbs_binned_counts_nd(gbs_net_t net, const int64_t *m_offset, double *P_mP, d
         if (dst[q])
             GBS_CUDA_TRY(cudaMemcpyAsync(dst[q], net->d_out2 + q * grid, sizeof(double) * grid,
                                          cudaMemcpyDeviceToHost, net->stream));
+    unsigned long long timed_out = 0;
+    GBS_CUDA_TRY(cudaMemcpyAsync(&timed_out, net->d_flags + 1, sizeof(timed_out),
+                                 cudaMemcpyDeviceToHost, net->stream));
     GBS_CUDA_TRY(cudaStreamSynchronize(net->stream));
+    if (timed_out) {
+        GBS_CUDA_TRY(cudaMemsetAsync(net->d_flags + 1, 0, sizeof(unsigned long long), net->stream));
+        return set_error(GBS_ETIMEOUT, "a GEMM or generating-function kernel gave up waiting on its pipeline");
+    }
     return GBS_OK;
 }
 
