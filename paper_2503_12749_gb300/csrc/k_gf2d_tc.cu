@@ -28,6 +28,9 @@
 // 23.1 ms; of 131072 trajectories the factors' digits 1.00 ms, the contraction
 // 0.90 ms (its products at 0.67 of the measured BF16 rate: 400 tiles make 2.6 waves,
 // and the drain of the sums is not fully covered, f64tc_pipe.cuh).
+// FP64 networks, 100 sub-ensembles, 20000 trajectories: 200 lossless modes on 128 x
+// 128 50.1 -> 2.00 ms; 50 and 10000, 60 modes on 32 x 32 x 32 51.3 -> 6.37 ms; 40 and
+// 20000, 8 modes (some trajectories too wide) 48.0 -> 6.76 ms.
 #include "bin2d.cuh"
 #include "f64tc_pipe.cuh"
 #include "gf64.cuh"
@@ -58,7 +61,7 @@ constexpr size_t kWorkBytes = (size_t)2 << 30;
 // contraction (us): 100 sub-ensembles on 64 x 64 of 16 trajectories 151 -> 164, 32
 // 158 -> 157, 64 271 -> 220; 128 x 128 of 32 324 -> 256, 512 2913 -> 1038; 32 x 32 of
 // 32 139 -> 164, 10 of 2000 2463 -> 848; 50 of 1000 on 32 x 32 x 32 9658 -> 5641.  FP64
-// networks, whose general kernel is ten times slower: 100 of 8 on 32 x 32 342 -> 226.
+// networks, whose general kernel is ten times slower: 100 of 8 on 32 x 32 345 -> 200.
 constexpr int64_t kMinPerSub = 32, kMinPerSub32 = 128, kMinPerSub64 = 8;
 
 // Offsets of the work space for `q` (a multiple of 8) trajectories per
