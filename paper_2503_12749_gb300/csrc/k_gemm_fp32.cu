@@ -30,7 +30,6 @@ constexpr int kStageFloats = kKT * 128;       // one operand's
 constexpr int kStageBytes = 2 * kStageFloats * 4;
 constexpr int kStages = 4;
 constexpr int kSmemBytes = kStages * kStageBytes + 128;
-constexpr uint64_t kWaitNs = 2000000000ull;
 static_assert(16 * kTS * 16 <= kStages * kStageBytes, "reduction buffer in the ring");
 
 __device__ __forceinline__ void fma2(float2 &acc, float2 a, float2 b) {
@@ -49,10 +48,11 @@ __device__ __forceinline__ void fma2(float2 &acc, float2 a, float2 b) {
 __global__ void __launch_bounds__(256, 2)
     k_gemm_fp32(const float *__restrict__ A, const float *__restrict__ B, int KB, int mtiles,
                 int64_t count, int64_t ld_part, double2 *__restrict__ nS_part, OccOut64 occ,
-                unsigned long long *err_ptr) {
+                uint64_t wait_ns, unsigned long long *err_ptr) {
     extern __shared__ __align__(128) uint8_t smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);
     uint64_t *empty = full + kStages;
+    uint64_t *never = empty + kStages;
     volatile unsigned long long *err = err_ptr;
     const int tid = threadIdx.x, lane = tid & 31;
     const int tx = tid & 15;  // 4 trajectories
@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(256, 2)
             ptx::mbar_init(ptx::smem_u32(&full[s]), 1);
             ptx::mbar_init(ptx::smem_u32(&empty[s]), 8);  // one arrival per warp
         }
+        ptx::mbar_init(ptx::smem_u32(never), 1);  // nothing arrives on it
         ptx::fence_barrier_init();
     }
     __syncthreads();
@@ -77,8 +78,9 @@ __global__ void __launch_bounds__(256, 2)
         ptx::bulk_load(dst, a_src + (size_t)kb * kStageFloats, kStageBytes / 2, bar);
         ptx::bulk_load(dst + kStageBytes / 2, b_src + (size_t)kb * kStageFloats, kStageBytes / 2, bar);
     };
+    int issued = min(KB, kStages);  // stages that thread 0 has loaded
     if (tid == 0)
-        for (int kb = 0; kb < min(KB, kStages); ++kb) load(kb);
+        for (int kb = 0; kb < issued; ++kb) load(kb);
 
     float2 acc[8][4];  // [row][alpha pair 0, 1, beta pair 0, 1]
 #pragma unroll
@@ -86,10 +88,16 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
 
-    for (int kb = 0; kb < KB; ++kb) {
+    // A warp whose wait gives up (wait_ns; the network's flag is raised) takes no
+    // further stage; its missing arrivals stop the loads.  With wait_ns = 0 the
+    // first wait is on a barrier that nothing arrives on.
+    bool ok = true;
+    if (wait_ns == 0ull) ok = __all_sync(0xffffffffu, ptx::mbar_wait(ptx::smem_u32(never), 0u, err, 0ull));
+    for (int kb = 0; ok && kb < KB; ++kb) {
         const int s = kb % kStages;
         const uint32_t ph = (uint32_t)(kb / kStages) & 1u;
-        ptx::mbar_wait(ptx::smem_u32(&full[s]), ph, err, kWaitNs);
+        ok = __all_sync(0xffffffffu, ptx::mbar_wait(ptx::smem_u32(&full[s]), ph, err, wait_ns));
+        if (!ok) break;
         const float *As = reinterpret_cast<const float *>(smem + s * kStageBytes) + ty * 8;
         const float *Bs = reinterpret_cast<const float *>(smem + s * kStageBytes) + kStageFloats + tx * 4;
 #pragma unroll
@@ -108,13 +116,21 @@ __global__ void __launch_bounds__(256, 2)
         }
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&empty[s]));
-        if (tid == 0 && kb + kStages < KB) {
-            ptx::mbar_wait(ptx::smem_u32(&empty[s]), ph, err, kWaitNs);
+        // (a stage after one that was not loaded is not either: `issued` counts them)
+        if (tid == 0 && kb + kStages < KB && issued == kb + kStages &&
+            ptx::mbar_wait(ptx::smem_u32(&empty[s]), ph, err, wait_ns)) {
             load(kb + kStages);
+            ++issued;
         }
         __syncwarp();
     }
-    __syncthreads();  // the ring is read; every load was waited for
+    // the ring becomes the reduction buffer, and another block's memory when this
+    // one exits: every load issued here has landed first, given up or not
+    if (tid == 0)
+        for (int kb = max(0, issued - kStages); kb < issued; ++kb)
+            ptx::mbar_wait(ptx::smem_u32(&full[kb % kStages]), (uint32_t)(kb / kStages) & 1u, err,
+                           200000000ull, false);
+    __syncthreads();  // and every warp has left it
 
     // occupations of this thread's 4 modes x 4 trajectories
     double2 *red = reinterpret_cast<double2 *>(smem);  // [16][kTS]
@@ -189,7 +205,7 @@ int launch_gemm_fp32(gbs_net *net, int64_t count, OccOut64 occ) {
     if (blocks > 0x7fffffff) return set_error(GBS_EINVAL, "chunk too large");
     k_gemm_fp32<<<(unsigned)blocks, 256, kSmemBytes, net->stream>>>(
         net->d_T32, static_cast<const float *>(net->d_B), (net->N + kKT - 1) / kKT, net->mtiles,
-        count, net->chunk, net->d_nS_part, occ, net->d_flags + 1);
+        count, net->chunk, net->d_nS_part, occ, net->wait_ns, net->d_flags + 1);
     GBS_LAUNCH_CHECK();
     return GBS_OK;
 }
