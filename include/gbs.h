@@ -402,15 +402,17 @@ int gbs_set_pair_autotune(int enable);
 
 /*
  * gbs_set_wait_limit -- bound, in nanoseconds, of every pipeline wait in the
- * network's tcgen05 GEMM launches (default 2e9; a wait that has not seen its
- * phase complete after that long raises the network's timeout flag, the
- * kernel stops issuing work, waits for what it already issued and returns).
- * The next synchronous read (gbs_binned_counts, gbs_check_finite,
- * gbs_moments) then returns GBS_ETIMEOUT and clears the flag; the sums of a
- * call that timed out are not meaningful (gbs_reset clears them).  A limit
- * of 0 exercises that path without a fault: each GEMM launch then first
- * waits on a barrier that nothing arrives on, gives up at once and issues
- * no MMA.  EINVAL: NULL network.
+ * network's GEMM launches and in the contractions of its joint generating
+ * functions (default 2e9; FP64 networks of fewer than 16 input modes, or
+ * outside the tensor cores' range, run a GEMM that waits for nothing).  A wait
+ * that has not seen its phase complete after that long raises the network's
+ * timeout flag; the kernel stops issuing work, waits for what it already
+ * issued and returns.  The next synchronous read (gbs_binned_counts,
+ * gbs_binned_counts_nd, gbs_check_finite, gbs_moments) then returns
+ * GBS_ETIMEOUT and clears the flag; the sums of a call that timed out are not
+ * meaningful (gbs_reset clears them).  A limit of 0 exercises that path
+ * without a fault: each such launch then first waits on a barrier that nothing
+ * arrives on, gives up at once and issues no product.  EINVAL: NULL network.
  */
 int gbs_set_wait_limit(gbs_net_t net, uint64_t limit_ns);
 

@@ -20,8 +20,6 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;  // warp 0 loads, warp 1 issues th
 constexpr int kBarBytes = 256;
 constexpr int kPipeBytes = 1024 + kStages * kStageBytes + kBarBytes;  // (the base is aligned to 1024)
 static_assert(kChunkKB == 2 * kBurst, "a chunk is two turns of each sub-tile");
-// bound of every pipeline wait (gbs_set_wait_limit is for the BF16 paths)
-constexpr uint64_t kWaitNs = 2000000000ull;
 
 // K-major operand without swizzle: core matrices of 8 rows x 16 bytes; the
 // two of a 16-wide K step 128 bytes apart (leading offset), 8-row groups 256
@@ -82,7 +80,8 @@ struct Pipe {
     __device__ __forceinline__ uint32_t tfull(int sub) const { return bar(2 * kStages + sub); }
     __device__ __forceinline__ uint32_t tempty(int sub) const { return bar(2 * kStages + 2 + sub); }
     __device__ __forceinline__ uint32_t drain() const { return bar(2 * kStages + 4); }
-    __device__ __forceinline__ uint32_t tmem_slot() const { return bar(2 * kStages + 5); }
+    __device__ __forceinline__ uint32_t never() const { return bar(2 * kStages + 5); }
+    __device__ __forceinline__ uint32_t tmem_slot() const { return bar(2 * kStages + 6); }
 
     // Barriers and TMEM; all threads; returns the TMEM base.
     __device__ __forceinline__ uint32_t open() {
@@ -96,6 +95,7 @@ struct Pipe {
                 ptx::mbar_init(tempty(b), kEpiWarps / 2);
             }
             ptx::mbar_init(drain(), 1);
+            ptx::mbar_init(never(), 1);  // nothing arrives on it
             ptx::fence_barrier_init();
         }
         if (threadIdx.x >> 5 == 1) {
@@ -117,6 +117,8 @@ struct Pipe {
         if (threadIdx.x >> 5 == 1) ptx::tmem_dealloc<1>(tmem, 512);
     }
 
+    // Waits are bounded by wait_ns (the network's, gbs_set_wait_limit); one that
+    // gives up raises *err and every role stops waiting.
     // One thread: the stages of contractions job(0, c), job(1, c), .. (false: no
     // more).
     template <typename Job>
@@ -162,6 +164,9 @@ struct Pipe {
             uint32_t base_ph = 0; // its phase
             uint32_t ck = 0;      // chunks issued so far
             bool ok = true;
+            // a wait limit of 0 asks for the timeout path itself: the first wait
+            // gives up (raising the flag) before any product is issued
+            if (wait_ns == 0ull) ok = ptx::mbar_wait(never(), 0u, err, 0ull);
             Contraction c;
             for (int i = 0; ok && job(i, c); ++i) {
                 const int KB = c.KB;

@@ -256,7 +256,7 @@ int launch_gemm_f64tc(gbs_net *net, int64_t count, OccOut64 occ) {
     const int grid = (int)std::min<int64_t>(ntiles, net->sm_count);
     k_gemm_f64tc<<<grid, kThreads, kSmemBytes, net->stream>>>(
         net->d_Aq, static_cast<const uint8_t *>(net->d_B), net->d_rowexp, f64tc_kblocks(net->N),
-        net->M, net->mtiles, (int)stiles, count, net->chunk, net->d_nS_part, occ, kWaitNs,
+        net->M, net->mtiles, (int)stiles, count, net->chunk, net->d_nS_part, occ, net->wait_ns,
         net->d_flags + 1);
     GBS_LAUNCH_CHECK();
     return GBS_OK;

@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kDigThreads)
 __global__ void __launch_bounds__(kThreads, 1)
     k_gf2d_tc(const uint8_t *__restrict__ imgA, const uint8_t *__restrict__ imgB,
               const SepMeta *__restrict__ meta, int q, const int *__restrict__ wmax, const GridD g,
-              int n_sub, double *__restrict__ acc, unsigned long long *err_ptr) {
+              int n_sub, double *__restrict__ acc, uint64_t wait_ns, unsigned long long *err_ptr) {
     extern __shared__ uint8_t smem_raw[];
     Pipe pipe(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -439,9 +439,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         return true;
     };
     if (warp == 0) {
-        if (lane == 0) pipe.load(job, err, kWaitNs);
+        if (lane == 0) pipe.load(job, err, wait_ns);
     } else if (warp == 1) {
-        if (lane == 0) pipe.multiply(job, tmem, err, kWaitNs);
+        if (lane == 0) pipe.multiply(job, tmem, err, wait_ns);
     } else {
         const int quarter = warp & 3, sub = (warp - 2) >> 2;
         const int row = quarter * 32 + lane;
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int part = 0; part < 2; ++part) {
                 const int blocks = ((part ? meta[r].x : meta[r].a) + kEntryBlock - 1) / kEntryBlock;
                 for (int n = (blocks + kChunkKB - 1) / kChunkKB; n > 0; --n, ++ck)
-                    pipe.add_chunk(ck, sub, tb, hi, lo, err, kWaitNs);
+                    pipe.add_chunk(ck, sub, tb, hi, lo, err, wait_ns);
                 // everything else is formed here: the sums leave it no registers
                 const int rem = t - r * mt * ct;
                 const int slot = rem / ct * kSlotTile + (row >> 1);
@@ -535,7 +535,7 @@ int launch_gf2d_tc(gbs_net *net, const GridD &g, const SepTrajT<V> *sep, int64_t
                           ((KB + kSlotTile - 1) / kSlotTile);
     k_gf2d_tc<<<(unsigned)std::min<int64_t>(tiles, net->sm_count), kThreads, kPipeBytes, net->stream>>>(
         base, base + w.img_b, m, w.q, net->d_wmax2, g, n_sub, reinterpret_cast<double *>(net->d_acc2),
-        net->d_flags + 1);
+        net->wait_ns, net->d_flags + 1);
     GBS_LAUNCH_CHECK();
     *rest = lists + 3 * (size_t)w.q;
     *meta = m;
