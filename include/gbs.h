@@ -225,7 +225,8 @@ int gbs_binned_counts_2d(gbs_net_t net, int64_t m1_offset, int64_t m2_offset, do
  * Independent of the sub-ensemble sums of gbs_sample (nothing accumulates
  * across calls).  Per trajectory and mode in FP32 on the BF16 paths (FP64
  * for magnitudes |n'| > 40), FP64 on the FP64 path; sums in FP64.
- * Unbinned networks only.  Synchronises.  Errors: EINVAL, ENOMEM, ECUDA.
+ * Unbinned networks only.  Synchronises.  Errors: EINVAL, ENOMEM, ECUDA,
+ * ETIMEOUT.
  */
 int gbs_moments(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E, int n_sub,
                 int mmax, int cmax, double *mom, double *sig_mom, double *marg, double *sig_marg);
@@ -312,7 +313,8 @@ int gbs_check_finite(gbs_net_t net, int64_t *count);
  * e0 .. e0+count-1 of key `seed`, computed by the same kernels as gbs_sample
  * (for parity tests): n[count] (input total sum_j alpha_j beta_j) and
  * nS[2*count] (output total sum_i alpha'_i beta'_i as (re, im)), host
- * buffers.  Does not touch the sub-ensemble sums.  Synchronises.
+ * buffers.  Does not touch the sub-ensemble sums.  Synchronises.  Errors:
+ * EINVAL, ECUDA, ETIMEOUT.
  */
 int gbs_debug_samples(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, double *n,
                       double *nS);
@@ -327,7 +329,7 @@ int gbs_debug_samples(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, 
  * (GBS_FP64) or 2^-47 (the BF16 split paths, whose double-float evaluation
  * rounds terms of order one to 2^-46).
  * Needs K1 fixed by a gbs_sample call.  Does not touch the sub-ensemble
- * sums.  Synchronises.  Errors: EINVAL, ECUDA.
+ * sums.  Synchronises.  Errors: EINVAL, ECUDA, ETIMEOUT.
  */
 int gbs_debug_windows(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, int *w);
 
@@ -336,7 +338,8 @@ int gbs_debug_windows(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, 
  * ("Applications to GBS") of trajectories e0 .. e0+count-1, as written by
  * the propagation GEMM's epilogue for gbs_moments: occ, host,
  * [M][count] complex as (re, im) pairs (FP32 values on the BF16 paths).
- * Unbinned networks only.  Synchronises.  Errors: EINVAL, ENOMEM, ECUDA.
+ * Unbinned networks only.  Synchronises.  Errors: EINVAL, ENOMEM, ECUDA,
+ * ETIMEOUT.
  */
 int gbs_debug_occupations(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, double *occ);
 
@@ -346,7 +349,8 @@ int gbs_debug_occupations(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t cou
  * matrix-P, 1 = +P; each the SUM of G(z_k) over the sub-ensemble's
  * trajectories) and counts[n_sub] (trajectories per sub-ensemble).  Used for
  * checkpoint/resume and to combine runs.  gbs_set_accumulators also fixes
- * (n_sub, K1) like a first gbs_sample.  Both synchronise.
+ * (n_sub, K1) like a first gbs_sample.  Both synchronise.  ETIMEOUT: the
+ * sums hold a launch that gave up waiting (gbs_set_wait_limit).
  */
 int gbs_get_accumulators(gbs_net_t net, int *n_sub, int *K1, double *acc, int64_t *counts);
 int gbs_set_accumulators(gbs_net_t net, int n_sub, int K1, const double *acc,
@@ -407,10 +411,11 @@ int gbs_set_pair_autotune(int enable);
  * outside the tensor cores' range, run a GEMM that waits for nothing).  A wait
  * that has not seen its phase complete after that long raises the network's
  * timeout flag; the kernel stops issuing work, waits for what it already
- * issued and returns.  The next synchronous read (gbs_binned_counts,
- * gbs_binned_counts_nd, gbs_check_finite, gbs_moments) then returns
- * GBS_ETIMEOUT and clears the flag; the sums of a call that timed out are not
- * meaningful (gbs_reset clears them).  A limit of 0 exercises that path
+ * issued and returns.  The next call that returns sampled data
+ * (gbs_binned_counts, gbs_binned_counts_nd, gbs_check_finite, gbs_moments,
+ * gbs_histogram, gbs_get_accumulators with acc, gbs_debug_samples / _windows /
+ * _occupations) then returns GBS_ETIMEOUT and clears the flag; the sums of a
+ * call that timed out are not meaningful (gbs_reset clears them).  A limit of 0 exercises that path
  * without a fault: each such launch then first waits on a barrier that nothing
  * arrives on, gives up at once and issues no product.  EINVAL: NULL network.
  */

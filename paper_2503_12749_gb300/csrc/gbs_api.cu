@@ -456,6 +456,23 @@ int validate_net(gbs_net *net) {
     return GBS_OK;
 }
 
+// The network's timeout flag (a kernel gave up waiting on its pipeline since the
+// last read).  Every entry point that returns sampled data queues its copy with
+// that of the data and reports it after the synchronisation.
+int queue_timeout_read(gbs_net *net, unsigned long long *flag) {
+    GBS_CUDA_TRY(cudaMemcpyAsync(flag, net->d_flags + 1, sizeof(*flag), cudaMemcpyDeviceToHost,
+                                 net->stream));
+    return GBS_OK;
+}
+
+int report_timeout(gbs_net *net, unsigned long long flag) {
+    if (!flag) return GBS_OK;
+    GBS_CUDA_TRY(cudaMemsetAsync(net->d_flags + 1, 0, sizeof(flag), net->stream));
+    GBS_CUDA_TRY(cudaStreamSynchronize(net->stream));
+    return set_error(GBS_ETIMEOUT, "a kernel gave up waiting on its pipeline; what was sampled since "
+                                   "the last check is not meaningful");
+}
+
 }  // namespace
 
 int fix_estimator(gbs_net *net, int n_sub, int K1) {
@@ -857,17 +874,10 @@ int gbs_check_finite(gbs_net_t net, int64_t *count) {
     int rc;
     if ((rc = validate_net(net))) return rc;
     if (count) *count = 0;
-    // a GEMM launch that gave up waiting on its pipeline since the last check
     unsigned long long timed_out = 0;
-    GBS_CUDA_TRY(cudaMemcpyAsync(&timed_out, net->d_flags + 1, sizeof(timed_out),
-                                 cudaMemcpyDeviceToHost, net->stream));
+    if ((rc = queue_timeout_read(net, &timed_out))) return rc;
     GBS_CUDA_TRY(cudaStreamSynchronize(net->stream));
-    if (timed_out) {
-        GBS_CUDA_TRY(cudaMemsetAsync(net->d_flags + 1, 0, sizeof(unsigned long long), net->stream));
-        GBS_CUDA_TRY(cudaStreamSynchronize(net->stream));
-        return set_error(GBS_ETIMEOUT, "a GEMM kernel gave up waiting on its pipeline; the sums "
-                                       "since the last check are not meaningful");
-    }
+    if ((rc = report_timeout(net, timed_out))) return rc;
     if (!net->est_fixed) return GBS_OK;
     prof_mark(net, GBS_PHASE_INVERT, 0, true);
     if ((rc = launch_count_nonfinite(net))) return rc;
@@ -903,9 +913,11 @@ int gbs_debug_samples(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, 
     if (count < 0 || !n || !nS) return set_error(GBS_EINVAL, "bad count or NULL output");
     const int saved_K1 = net->K1;
     if (net->K1 == 0) net->K1 = 2;  // finalize computes windows for some K1; unused here
-    for (int64_t done = 0; done < count; done += net->chunk) {
+    unsigned long long timed_out = 0;
+    for (int64_t done = 0; done < count && !timed_out; done += net->chunk) {
         const int64_t c = std::min<int64_t>(net->chunk, count - done);
-        if ((rc = run_chunk_front(net, seed, e0 + (uint64_t)done, c))) {
+        if ((rc = run_chunk_front(net, seed, e0 + (uint64_t)done, c)) ||
+            (rc = queue_timeout_read(net, &timed_out))) {
             net->K1 = saved_K1;
             return rc;
         }
@@ -921,7 +933,7 @@ int gbs_debug_samples(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, 
         }
     }
     net->K1 = saved_K1;
-    return GBS_OK;
+    return report_timeout(net, timed_out);
 }
 
 int gbs_debug_windows(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, int *w) {
@@ -930,9 +942,12 @@ int gbs_debug_windows(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, 
     if (count < 0 || !w) return set_error(GBS_EINVAL, "bad count or NULL output");
     if (!net->est_fixed) return set_error(GBS_EINVAL, "K1 not fixed yet (call gbs_sample first)");
     static_assert(sizeof(Window) == 2 * sizeof(int), "window layout");
-    for (int64_t done = 0; done < count; done += net->chunk) {
+    unsigned long long timed_out = 0;
+    for (int64_t done = 0; done < count && !timed_out; done += net->chunk) {
         const int64_t c = std::min<int64_t>(net->chunk, count - done);
-        if ((rc = run_chunk_front(net, seed, e0 + (uint64_t)done, c))) return rc;
+        if ((rc = run_chunk_front(net, seed, e0 + (uint64_t)done, c)) ||
+            (rc = queue_timeout_read(net, &timed_out)))
+            return rc;
         cudaError_t e1 = cudaMemcpyAsync(w + 2 * done, net->d_win, sizeof(Window) * c,
                                          cudaMemcpyDeviceToHost, net->stream);
         cudaError_t e2 = cudaStreamSynchronize(net->stream);
@@ -940,7 +955,7 @@ int gbs_debug_windows(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t count, 
             return set_error(GBS_ECUDA, "debug copy failed: %s",
                              cudaGetErrorString(e2 != cudaSuccess ? e2 : e1));
     }
-    return GBS_OK;
+    return report_timeout(net, timed_out);
 }
 
 int gbs_histogram(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E, const int *m,
@@ -977,13 +992,15 @@ int gbs_histogram(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E
         if (!rc) rc = launch_histogram(net, c, spec, d_cnt);
     }
     net->K1 = saved_K1;
+    unsigned long long timed_out = 0;
+    if (!rc) rc = queue_timeout_read(net, &timed_out);
     if (!rc) {
         std::vector<unsigned long long> h(total);
         if (cudaMemcpyAsync(h.data(), d_cnt, total * sizeof(unsigned long long),
                             cudaMemcpyDeviceToHost, net->stream) != cudaSuccess ||
             cudaStreamSynchronize(net->stream) != cudaSuccess)
             rc = set_error(GBS_ECUDA, "histogram copy failed");
-        else
+        else if (!(rc = report_timeout(net, timed_out)))
             for (size_t q = 0; q < total; ++q) counts[q] = (int64_t)h[q];
     }
     net_free(net, d_cnt);
@@ -1051,9 +1068,11 @@ int gbs_debug_occupations(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t cou
     if (rc) return rc;
     const size_t elt = fp64 ? sizeof(double) : sizeof(float);
     std::vector<uint8_t> h((size_t)2 * plane * elt);
+    unsigned long long timed_out = 0;
     for (int64_t done = 0; !rc && done < count; done += ld) {
         const int64_t c = std::min<int64_t>(ld, count - done);
         rc = run_chunk_occ(net, seed, e0 + (uint64_t)done, c, d_occ, ld);
+        if (!rc) rc = queue_timeout_read(net, &timed_out);
         if (rc) break;
         if (cudaMemcpyAsync(h.data(), d_occ, h.size(), cudaMemcpyDeviceToHost, net->stream) !=
                 cudaSuccess ||
@@ -1061,6 +1080,7 @@ int gbs_debug_occupations(gbs_net_t net, uint64_t seed, uint64_t e0, int64_t cou
             rc = set_error(GBS_ECUDA, "occupation copy failed");
             break;
         }
+        if ((rc = report_timeout(net, timed_out))) break;
         for (int j = 0; j < net->M; ++j)
             for (int64_t i = 0; i < c; ++i) {
                 const size_t a = (size_t)j * ld + i, b = (size_t)plane + a;
@@ -1154,17 +1174,12 @@ int gbs_moments(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E, 
     if (!rc) {
         std::vector<double> h(2 * nm + 2 * nc);
         unsigned long long timed_out = 0;
-        if (cudaMemcpyAsync(h.data(), d_out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost,
-                            net->stream) != cudaSuccess ||
-            cudaMemcpyAsync(&timed_out, net->d_flags + 1, sizeof(timed_out), cudaMemcpyDeviceToHost,
+        if (queue_timeout_read(net, &timed_out) ||
+            cudaMemcpyAsync(h.data(), d_out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost,
                             net->stream) != cudaSuccess ||
             cudaStreamSynchronize(net->stream) != cudaSuccess)
             rc = set_error(GBS_ECUDA, "moment copy failed");
-        else if (timed_out) {
-            cudaMemsetAsync(net->d_flags + 1, 0, sizeof(unsigned long long), net->stream);
-            cudaStreamSynchronize(net->stream);
-            rc = set_error(GBS_ETIMEOUT, "a GEMM or moments kernel gave up waiting on its pipeline");
-        } else {
+        else if (!(rc = report_timeout(net, timed_out))) {
             if (mom) std::memcpy(mom, h.data(), sizeof(double) * nm);
             if (sig_mom) std::memcpy(sig_mom, h.data() + nm, sizeof(double) * nm);
             if (marg) std::memcpy(marg, h.data() + 2 * nm, sizeof(double) * nc);
@@ -1186,10 +1201,14 @@ int gbs_get_accumulators(gbs_net_t net, int *n_sub, int *K1, double *acc, int64_
     if (n_sub) *n_sub = net->n_sub;
     if (K1) *K1 = net->K1;
     if (!net->est_fixed) return GBS_OK;
-    if (acc)
+    unsigned long long timed_out = 0;
+    if (acc) {
+        if ((rc = queue_timeout_read(net, &timed_out))) return rc;
         GBS_CUDA_TRY(cudaMemcpyAsync(acc, net->d_acc, sizeof(double2) * 2 * net->n_sub * net->K1,
                                      cudaMemcpyDeviceToHost, net->stream));
+    }
     GBS_CUDA_TRY(cudaStreamSynchronize(net->stream));
+    if ((rc = report_timeout(net, timed_out))) return rc;
     if (counts) std::memcpy(counts, net->counts.data(), sizeof(int64_t) * net->n_sub);
     return GBS_OK;
 }
@@ -1276,14 +1295,9 @@ int gbs_binned_counts_nd(gbs_net_t net, const int64_t *m_offset, double *P_mP, d
             GBS_CUDA_TRY(cudaMemcpyAsync(dst[q], net->d_out2 + q * grid, sizeof(double) * grid,
                                          cudaMemcpyDeviceToHost, net->stream));
     unsigned long long timed_out = 0;
-    GBS_CUDA_TRY(cudaMemcpyAsync(&timed_out, net->d_flags + 1, sizeof(timed_out),
-                                 cudaMemcpyDeviceToHost, net->stream));
+    if ((rc = queue_timeout_read(net, &timed_out))) return rc;
     GBS_CUDA_TRY(cudaStreamSynchronize(net->stream));
-    if (timed_out) {
-        GBS_CUDA_TRY(cudaMemsetAsync(net->d_flags + 1, 0, sizeof(unsigned long long), net->stream));
-        return set_error(GBS_ETIMEOUT, "a GEMM or generating-function kernel gave up waiting on its pipeline");
-    }
-    return GBS_OK;
+    return report_timeout(net, timed_out);
 }
 
 int gbs_sample_2d(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E, int n_sub,
