@@ -157,8 +157,15 @@ int gbs_make_network_binned(int N, int M, const double *T, const double *r, cons
  * with the exponent summed over the bins), summed per sub-ensemble (e mod
  * n_sub).  K: host, d powers of two >= 2 with prod K_b <= 2^22; the first
  * call fixes (n_sub, K) until gbs_reset.  Generating functions in FP64 (FP64
- * networks) or double-float (BF16 networks), summed in FP64.  Errors: EINVAL
- * (not a binned network, sizes), ENOMEM, ECUDA.
+ * and FP32 networks) or double-float (BF16 networks), summed in FP64.  Calls of
+ * 8 (FP64, FP32) or 32 to 128 (BF16) and more trajectories per sub-ensemble on
+ * grids of at least 32 points in the last dimension and 32 in the others
+ * together contract the two factors of exp(sum_b (z_b-1) n_Sb) as fixed-point
+ * numbers of 56 bits, exact sums of factors rounded to 2^-53 (FP64) or
+ * 2^-47 of the sub-ensemble's largest.  They take up to 2 GiB of work space from
+ * the device's memory pool for the duration of the call; where it has none to
+ * spare the call runs on the general kernels, whose sums round differently.
+ * Errors: EINVAL (not a binned network, sizes), ENOMEM, ECUDA.
  */
 int gbs_sample_nd(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E, int n_sub,
                   const int *K);
@@ -186,9 +193,8 @@ int gbs_binned_counts_nd(gbs_net_t net, const int64_t *m_offset, double *P_mP, d
  * z_b = exp(2 pi i k_b / K_b) (the one-bin form of Eq. c-number-variable
  * with the exponent summed over the bins), summed per sub-ensemble (e mod
  * n_sub).  K1, K2: powers of two, K1 K2 <= 2^22; the first call fixes
- * (n_sub, K1, K2) until gbs_reset.  Generating functions in FP64 (FP64
- * networks) or double-float (BF16 networks), summed in FP64.  Errors: EINVAL
- * (not a network of two bins, sizes), ENOMEM, ECUDA.
+ * (n_sub, K1, K2) until gbs_reset.  Errors: EINVAL (not a network of two
+ * bins, sizes), ENOMEM, ECUDA.
  */
 int gbs_sample_2d(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E, int n_sub,
                   int K1, int K2);

@@ -191,8 +191,6 @@ void release_estimator(gbs_net *net) {
     net_free(net, net->d_out2);
     net_free(net, net->d_mo2);
     pool_free(net->d_sep2, net->stream);
-    pool_free(net->d_gf2, net->stream);
-    net->gf2_bytes = 0;
     net->counts2.clear();
     net->est2_fixed = false;
     net->n_sub2 = 0;
@@ -1240,7 +1238,13 @@ int gbs_sample_nd(gbs_net_t net, uint64_t seed, uint64_t first_sample, int64_t E
     if (first_sample + (uint64_t)E < first_sample)
         return set_error(GBS_EINVAL, "sample index range overflows 64 bits");
     if ((rc = fix_estimator2d(net, n_sub, K))) return rc;
-    if (fold_sampler(net, E, net->chunk)) {
+    struct WorkSpace {  // of the joint generating functions, for this call
+        gbs_net *net;
+        ~WorkSpace() { release_gf2d_tc(net); }
+    } work{net};
+    const bool fold = fold_sampler(net, E, net->chunk);
+    if ((rc = reserve_gf2d_tc(net, E))) return rc;
+    if (fold) {
         auto gemm = [&](int64_t c, const SampleJob &job) {
             return job.count ? launch_gemm_tc_sampling(net, c, job) : launch_gemm_tc(net, c);
         };

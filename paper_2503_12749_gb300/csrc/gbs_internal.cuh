@@ -253,7 +253,8 @@ struct gbs_net {
     double *d_out2 = nullptr;       // [4][grid2]
     int64_t *d_mo2 = nullptr;       // [kMaxBins] DFT window offsets
     void *d_sep2 = nullptr;         // [chunk] per-trajectory constants
-    void *d_gf2 = nullptr;          // work space of the digit-product kernels (k_gf2d_tc.cu)
+    void *d_gf2 = nullptr;          // work space of the digit-product kernels (k_gf2d_tc.cu),
+                                    // during a gbs_sample_nd call
     size_t gf2_bytes = 0;
 };
 
@@ -436,6 +437,8 @@ int launch_moment_stats(const MomentSpec &sp, bool fp64, const double *acc, cons
 // inversion into out_dev[4][grid2] (*launches: kernels launched).
 int launch_finalize2d(gbs_net *net, int64_t count);
 int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count, int *launches);
+int reserve_gf2d_tc(gbs_net *net, int64_t E);
+void release_gf2d_tc(gbs_net *net);
 size_t sep2_bytes_per_trajectory();
 int launch_tables2d(gbs_net *net);
 int launch_invert2d(gbs_net *net, const int64_t *m_off, double *out_dev, int *launches);

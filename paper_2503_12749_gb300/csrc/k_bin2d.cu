@@ -796,18 +796,35 @@ int launch_finalize2d(gbs_net *net, int64_t count) {
     return GBS_OK;
 }
 
-// Work space of the digit-product kernels; ENOTSUP where the device has none to
-// spare (the outer-product kernel needs none).
-int reserve_gf2d_tc(gbs_net *net, int64_t KA, int KB, int64_t count) {
-    size_t bytes = 0;
-    gf2d_tc_piece(net->n_sub2, KA, KB, count, &bytes);
-    if (bytes <= net->gf2_bytes) return GBS_OK;
+// Work space of the digit-product kernels for one call of E trajectories in chunks
+// of net->chunk, from the pool and given back to it by release_gf2d_tc: nothing is
+// allocated between a call's launches, none stays with the network, and inside a
+// stream capture the allocation and its release belong to the graph.  A device
+// that has none to spare runs the call on the outer-product kernels, which need
+// none (and round differently).
+int reserve_gf2d_tc(gbs_net *net, int64_t E) {
+    const bool fp64 = simt_precision(net->precision);
+    const int KB = net->Kd[net->nbins - 1];
+    const int64_t KA = net->grid2 / KB;
+    size_t most = 0;
+    // a whole chunk's, the last chunk's (pieces of equal size: neither bounds the other)
+    for (int64_t count : {std::min(E, net->chunk), E % net->chunk}) {
+        size_t bytes = 0;
+        if (count > 0 && gf2d_tc_takes(fp64, net->n_sub2, KA, KB, count))
+            gf2d_tc_piece(net->n_sub2, KA, KB, count, &bytes);
+        most = std::max(most, bytes);
+    }
+    if (!most) return GBS_OK;
+    const int rc = pool_alloc(&net->d_gf2, most, net->stream, "joint generating functions");
+    if (rc) return rc == GBS_ENOMEM ? GBS_OK : rc;
+    net->gf2_bytes = most;
+    return GBS_OK;
+}
+
+void release_gf2d_tc(gbs_net *net) {
     pool_free_raw(net->d_gf2, net->stream);
     net->d_gf2 = nullptr;
     net->gf2_bytes = 0;
-    if (pool_alloc(&net->d_gf2, bytes, net->stream, "joint generating functions")) return GBS_ENOTSUP;
-    net->gf2_bytes = bytes;
-    return GBS_OK;
 }
 
 int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count, int *launches) {
@@ -818,9 +835,8 @@ int launch_gf2d(gbs_net *net, uint64_t e0, int64_t count, int *launches) {
     const bool simt = simt_precision(net->precision);
     const int KB = net->Kd[net->nbins - 1];
     const int64_t KA = net->grid2 / KB;
-    int rc = GBS_ENOTSUP;
-    if (gf2d_tc_takes(simt, net->n_sub2, KA, KB, count)) rc = reserve_gf2d_tc(net, KA, KB, count);
-    const bool tc = rc == GBS_OK;
+    const bool tc = net->d_gf2 && gf2d_tc_takes(simt, net->n_sub2, KA, KB, count);
+    int rc = GBS_OK;
     SepTraj *sep = static_cast<SepTraj *>(net->d_sep2);
     SepTraj64 *sep64 = static_cast<SepTraj64 *>(net->d_sep2);
     if (tc || !simt) {
