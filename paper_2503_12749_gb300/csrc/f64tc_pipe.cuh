@@ -251,6 +251,9 @@ struct Pipe {
         const int lane = threadIdx.x & 31;
         // on a timeout the epilogue keeps going without waiting
         ptx::mbar_wait(tfull(sub), ck & 1u, err, wait_ns);
+        // the loads below are the whole warp's: lanes may come here apart, from the
+        // wait or from what a caller does for some rows only
+        __syncwarp();
         ptx::tc_fence_after();
         // 8 columns at a time: the sums hold 128 registers.  The other sub-tile's
         // turn (kBurst stages, 2176 clocks) covers this; the conversions' 16 lanes

@@ -315,6 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if constexpr (BN == kBNGrad) {
             // (every MMA has completed, so every load of the ring has been read)
             ptx::mbar_wait(ptx::smem_u32(tfull), 0u, err);
+            __syncwarp();  // the TMEM loads are the whole warp's
             ptx::tc_fence_after();
             for (int c0 = half; c0 < BN && n0 + c0 < p.cols_valid; c0 += 64) {
                 float v[32];
@@ -342,6 +343,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 __syncwarp();
             }
             ptx::mbar_wait(ptx::smem_u32(tfull), 0u, err);
+            __syncwarp();  // the TMEM loads are the whole warp's
             ptx::tc_fence_after();
             float v[32];
             ptx::tmem_ld32(tl + (uint32_t)half, v);
