@@ -48,10 +48,9 @@ constexpr int kFp64TileSamples = 32;            // samples per FP64 GEMM tile
 constexpr int kFp32TileSamples = 64;            // samples per FP32 GEMM tile
 constexpr int kFp32BlockK = 16;                 // input modes per FP32 GEMM stage
 // Input modes from which the FP64 GEMM runs as digit products on the tensor
-// cores (k_gemm_f64tc.cu): one whole K step.  It is the faster one at every
-// size (N = M = 16, 16384 trajectories: 0.049 against 0.150 ms), but its
-// error grows as sqrt(N) against the FMA chain's N, and below about 10 modes
-// the chain's is the smaller.
+// cores (k_gemm_f64tc.cu): one whole K step.  It is the faster one from there (16384
+// trajectories, N = M = 16: 0.043 against 0.149 ms) and the more accurate one
+// (k_gemm_f64tc.cu); smaller networks keep the FMA kernel (N = 15: 0.149 ms).
 constexpr int kF64tcMinN = 16;
 constexpr int kTcTileModes = 64;                // output modes per tcgen05 tile (128 A rows)
 constexpr int kTcTileSamples = 128;             // samples per tcgen05 tile (256 B rows)

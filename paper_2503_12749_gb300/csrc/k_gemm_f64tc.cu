@@ -9,30 +9,41 @@
 // of matrix multiplication and its applications", Numer. Algorithms 59, 2012,
 // in its fixed-point form):
 //   T_ij 2^{e_j - f_i} = 2^-55 sum_{p=0..6} a_p 2^{8 (6 - p)},   |a_p| <= 128,
-//   alpha_j 2^{-e_j}   = 2^-55 sum_{q=0..6} b_q 2^{8 (6 - q)},   |b_q| <= 128,
+//   alpha_j 2^{-e_j}   = 2^-58 sum_{q=0..6} b_q 2^{8 (6 - q)},   |b_q| <= 128, |b_0| <= 1024,
 //   D_d = sum_j sum_{p + q = d} a_p b_q   (d = 0..7),
-//   alpha'_i = 2^{f_i - 70} sum_d D_d 2^{8 (7 - d)}.
+//   alpha'_i = 2^{f_i - 73} sum_d D_d 2^{8 (7 - d)}.
 // e_j bounds |alpha_j|, |beta_j| for every possible draw (the Box-Muller
 // radius of a 53-bit uniform is below 8.67), f_i bounds row i of T 2^{e_j}.
-// A digit is an integer of at most 8 bits, so it is an FP16 number; 8 products
-// of at most 2^14 over 128 input modes sum to at most 2^24, so every FP32
-// accumulator value is an exact integer.  The accumulators are added to
-// 64-bit integers every 128 modes, so the only errors are the quantisation
-// of the operands (2^-56 of the bounds) and the digit pairs p + q >= 8
-// (below 2^-61 of them): for N input modes about 2 sqrt(N) 2^-54 of a typical
-// term against 0.6 N 2^-54 for a chain of FP64 FMAs.
+// A digit is an integer of at most 11 bits, so it is an FP16 number, and every FP32
+// accumulator value is an exact integer below 2^24 over 128 input modes (one
+// chunk): the products without b_0, d (of D_7: 6) of at most 2^21 per D_d, by their
+// bound; the one with it, a_d b_0 summed, because b_0 is Gaussian of standard
+// deviation below 118.2 (2^10 / 8.67), so that the sum over 128 modes has at most
+// 2^17.4 whatever T is and exceeds the 2^21 that D_1 leaves (the drain wants D_0 and
+// D_1 below 2^22) by 12.3 standard deviations, the 2^22 of the others by 24:
+// less than once in 1e33 sums.
+// The accumulators are added to 64-bit integers every 128 modes, so the only
+// errors are the quantisation of the operands (amplitudes above 1/32 of their
+// scale and entries of T above 1/8 of their row's largest are exact, smaller ones
+// err by 2^-59 and 2^-56 of it), the digit pairs p + q >= 8 (below 2^-64) and
+// the sum's rounding to 53 bits, against a rounding at every term of a chain of
+// FP64 FMAs.  So it is the more accurate one however few entries a row of T has;
+// kTrajBits = 0 was not (the figures in parentheses below).
 //
 // Why: GB300 has 2 FP64 FMA lanes per SM and clock (1.25 TFLOP/s) but 4096
 // 16-bit ones, so 34 exact 16-bit products cost a fiftieth of one FP64 product.
 // Measured (one GB300): N = M = 1000, 32768 trajectories 5.50 ms against 216.4
 // for the FP64 FMA kernel (34 products at 0.84 of the measured BF16 rate; 6.27 with
 // a conversion for every sum and 32 columns read at once, f64tc_pipe.cuh);
-// N = M = 16, 16384 trajectories 0.049 against 0.150.  Root mean square error of
+// N = M = 16, 16384 trajectories 0.043 against 0.149.  Root mean square error of
 // n_S against 113-bit arithmetic, relative to sum |alpha'_i| |beta'_i|, real and
-// imaginary part (the input samples' own rounding included): N = 16 1.21e-16 and
-// 1.9e-17 against 1.18e-16 and 4.0e-17, N = 64 7.6e-17 and 1.2e-17 against 1.09e-16
-// and 3.8e-17, N = 200 8.7e-17 and 5.8e-18 against 1.17e-16 and 4.0e-17, N = 400
-// 8.8e-17 and 4.5e-18 against 1.12e-16 and 3.7e-17.
+// imaginary part (the input samples' own rounding included): N = 16 9.8e-17 and
+// 2.2e-17 against 1.18e-16 and 4.0e-17, N = 64 7.6e-17 and 1.3e-17 against 1.09e-16
+// and 3.8e-17, N = 200 8.6e-17 and 5.4e-18 against 1.17e-16 and 4.0e-17, N = 400
+// 9.1e-17 and 4.4e-18 against 1.12e-16 and 3.7e-17.  Median relative error of an
+// occupation n'_i, N = 32, likewise: diagonal T 2.09e-16 against 2.11e-16 (3.2e-16
+// with kTrajBits = 0), blocks of 2 modes 1.90e-16 against 1.98e-16 (2.9e-16), of 4
+// 1.93e-16 against 2.10e-16 (2.8e-16), dense 2.03e-16 against 3.08e-16 (2.8e-16).
 //
 // Tile: 64 output modes (128 rows Re/Im) x 32 trajectories, as two sub-tiles
 // of 16 trajectories (16 alpha and 16 beta columns).  A sub-tile's eight D_d
@@ -132,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int k = 0; k < nchunk; ++k, ++ck) pipe.add_chunk(ck, sub, tb, hi, lo, err, wait_ns);
             // alpha' (columns 0..15) and beta' (16..31) of this row; the
             // partner lane holds the other of (Re, Im) of the same mode
-            const int f = row_exp[tl.mt * 128 + row] - 70;
+            const int f = row_exp[tl.mt * 128 + row] - 70 - kTrajBits;
             const bool odd = (lane & 1) != 0;
             // even lanes (Re rows) form the real parts ar br + ai bi, odd lanes
             // the imaginary parts ai br - ar bi

@@ -162,16 +162,16 @@ __global__ void __launch_bounds__(256, 2)
                             double a, b;
                             amplitudes(sh, seed, e, (uint32_t)j, sq[j], a, b);
                             sum[t >> 1] = fma(a, b, sum[t >> 1]);
-                            const int s = 55 - col_exp[j];
+                            const int s = 55 + kTrajBits - col_exp[j];
                             xa[h] = to_fixed(a, s);
                             xb[h] = to_fixed(b, s);
                         }
                     }
                     uint32_t w[kDigits];
-                    digit_pairs(xa[0], xa[1], w);
+                    digit_pairs<true>(xa[0], xa[1], w);
 #pragma unroll
                     for (int q = 0; q < kDigits; ++q) da[q][t >> 1] = w[q];
-                    digit_pairs(xb[0], xb[1], w);
+                    digit_pairs<true>(xb[0], xb[1], w);
 #pragma unroll
                     for (int q = 0; q < kDigits; ++q) db[q][t >> 1] = w[q];
                 }
