@@ -126,6 +126,14 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// a + b rounded, its rounding error added to err (TwoSum; Knuth, "The Art of
+// Computer Programming" 2, 4.2.2).
+__device__ __forceinline__ double two_sum(double a, double b, double &err) {
+    const double s = a + b, bb = s - a;
+    err += (a - (s - bb)) + (b - bb);
+    return s;
+}
+
 // ---------------------------------------------------------------------------
 // FP64 path on the tensor cores: the digit tiles of f64tc.cuh.  `wpg` of a
 // block's 8 warps (1, 2, 4 or 8, by the number of modes) hold 8 trajectories (one
@@ -139,7 +147,7 @@ __global__ void __launch_bounds__(256, 2)
                    uint64_t e0, int64_t count, uint8_t *__restrict__ B, double *__restrict__ n_out) {
     using namespace f64tc;
     __shared__ __align__(16) NormTab sh;
-    __shared__ double s_n[8][8];
+    __shared__ double s_n[8][8], s_err[8][8];
     load_tab(sh, tab);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int per = 8 / wpg * 8;  // trajectories per block and turn
@@ -185,20 +193,30 @@ __global__ void __launch_bounds__(256, 2)
                         make_uint4(db[q][0], db[q][1], db[q][2], db[q][3]);
                 }
             }
-        double part = (sum[0] + sum[1]) + (sum[2] + sum[3]);
-        part += __shfl_xor_sync(0xffffffffu, part, 8);
-        part += __shfl_xor_sync(0xffffffffu, part, 16);
-        if (lane < 8) s_n[warp][lane] = part;
+        // the last additions with their rounding errors, rounded once: they err the most
+        // of a pairwise sum, and an unequal last part adds one (N = 130: 8.5e-17 of sum
+        // |alpha beta| without, 7.4e-17 for 32 interleaved chains, 6.3e-17 so).  Where
+        // warps follow, theirs are enough, and the lanes' cost 0.5 % of a call at N = 1000.
+        double part = (sum[0] + sum[1]) + (sum[2] + sum[3]), err = 0.0;
+        if (wpg <= 2) {
+            part = two_sum(part, __shfl_xor_sync(0xffffffffu, part, 8), err);
+            err += __shfl_xor_sync(0xffffffffu, err, 16);
+            part = two_sum(part, __shfl_xor_sync(0xffffffffu, part, 16), err);
+        } else {
+            part += __shfl_xor_sync(0xffffffffu, part, 8);
+            part += __shfl_xor_sync(0xffffffffu, part, 16);
+        }
+        if (lane < 8) {
+            s_n[warp][lane] = part;
+            s_err[warp][lane] = err;
+        }
         __syncthreads();
-        // pairwise, as the shuffles: a chain of eight had 1.3 times its error
         if ((warp & (wpg - 1)) == 0 && lane < 8 && i < count) {
-            if (wpg == 1) {
-                n_out[i] = part;
-            } else {
-                double v[4];
-                for (int w = 0; w < wpg / 2; ++w) v[w] = s_n[warp + 2 * w][lane] + s_n[warp + 2 * w + 1][lane];
-                n_out[i] = wpg == 2 ? v[0] : wpg == 4 ? v[0] + v[1] : (v[0] + v[1]) + (v[2] + v[3]);
+            for (int w = 1; w < wpg; ++w) {
+                err += s_err[warp + w][lane];
+                part = two_sum(part, s_n[warp + w][lane], err);
             }
+            n_out[i] = part + err;
         }
         __syncthreads();
     }
