@@ -70,6 +70,13 @@ struct Ring {
         kStages * kStageBytes + (BN == kBN ? kEpiWarps * kTurnBytes : 0);
     static constexpr int kSmem = 1024 + kBarOffset + 256;
     static_assert(kSmem <= 227 * 1024, "shared memory of the MLP GEMM");
+    // accumulators side by side: the tensor core truncates its FP32 accumulator at
+    // every product, about 2^-24 of it, so a weight gradient's K (the batch) is
+    // summed in kAccs parts per CTA, which the epilogue adds.  Median error of a last
+    // layer's gradient, width 512, 1800 rows (3 splits): 6.7e-6 with one accumulator,
+    // 5.4e-6 with four (8 splits of one: 5.7e-6); 1024, 32768 rows: 1.1e-4 and 2.3e-5
+    // (2.3e-5).  10 Adam steps of 1800 rows 1473 -> 1488 us.
+    static constexpr int kAccs = BN == kBN ? 1 : 4;
 };
 constexpr int kThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 MMA, then the epilogue
 constexpr int kMaxLayers = 8;
@@ -210,6 +217,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile unsigned long long *err = p.err;
     const int kb0 = split * p.kb_split;
     const int nkb = min(p.kb_total, kb0 + p.kb_split) - kb0;  // >= 1 (host)
+    // 32-wide K blocks per accumulator
+    const int acc_blocks = (nkb * (kBK / 32) + R::kAccs - 1) / R::kAccs;
     const int m0 = blockIdx.x * kBM;
     const int n0 = blockIdx.y * BN;
 
@@ -223,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ptx::fence_barrier_init();
     }
     if (warp == 1) {
-        ptx::tmem_alloc(ptx::smem_u32(tmem_slot), BN);
+        ptx::tmem_alloc(ptx::smem_u32(tmem_slot), R::kAccs * BN);
         ptx::tmem_relinquish();
     }
     if (threadIdx.x == 0) {
@@ -284,17 +293,24 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ptx::tc_fence_after();
                 // per 32 K the correction products first, A0 B0 last
 #pragma unroll
-                for (int h = 0; h < kBK / 32; ++h)
+                for (int h = 0; h < kBK / 32; ++h) {
+                    uint32_t d = tmem_base;
+                    if (R::kAccs > 1) {
+                        const int block = kb * (kBK / 32) + h;
+                        d += (uint32_t)(block / acc_blocks * BN);
+                        if (block % acc_blocks == 0) acc = 0u;
+                    }
                     for (int pr = 0; pr < np; ++pr) {
                         const uint32_t a0 = ptx::smem_u32(a_tile(stage, pa[pr])) + h * 64;
                         const uint32_t b0 = ptx::smem_u32(b_tile(stage, pb[pr])) + h * 64;
 #pragma unroll
                         for (int kk = 0; kk < 2; ++kk) {
-                            ptx::mma_bf16(tmem_base, ptx::desc_k_sw128(a0 + kk * 32),
+                            ptx::mma_bf16(d, ptx::desc_k_sw128(a0 + kk * 32),
                                           ptx::desc_k_sw128(b0 + kk * 32), kIdesc, acc);
                             acc = 1u;
                         }
                     }
+                }
                 ptx::mma_commit(ptx::smem_u32(&empty[stage]));
                 if (++stage == kStages) {
                     stage = 0;
@@ -321,6 +337,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 float v[32];
                 ptx::tmem_ld32(tl + (uint32_t)c0, v);
                 ptx::tmem_ld_wait();
+                for (int b = acc_blocks, a = 1; b < nkb * (kBK / 32); b += acc_blocks, ++a) {
+                    float u[32];
+                    ptx::tmem_ld32(tl + (uint32_t)(a * BN + c0), u);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) v[i] += u[i];
+                }
                 turn_put(tb, lane, v);
                 store_block_f32(p.out + split * p.split_stride + (size_t)row0 * p.ld_out + n0 + c0,
                                 p.ld_out, tb, lane);
@@ -406,7 +429,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     if (warp == 1) {
         ptx::tc_fence_after();
-        ptx::tmem_dealloc(tmem_base, BN);
+        ptx::tmem_dealloc(tmem_base, R::kAccs * BN);
     }
 }
 
@@ -785,13 +808,14 @@ int plan_backward(gbs_mlp *m, Plan &plan, int batch) {
     }
     // weight gradients: dW_l = dY_l^T H_{l-1}, K = the batch, split so that the
     // launch is one wave: the hidden and output layers alike, the first (one
-    // column tile) from what they leave
+    // column tile) from what they leave; two splits at least, which with their
+    // accumulators sum the batch in eight parts, 32 rows being the smallest
     int sms = 0, tiles = 0;
     GBS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
     for (int l = 1; l < L; ++l)
         tiles += (m->lay.n_out[l] / kBM) * ((m->lay.k_pad[l] + kBNGrad - 1) / kBNGrad);
-    const int S = std::max(1, std::min(kMaxSplit, sms / tiles));
-    const int S0 = std::max(1, std::min(kMaxSplit, (sms - S * tiles) / (m->lay.n_out[0] / kBM)));
+    const int S = std::max(2, std::min(kMaxSplit, sms / tiles));
+    const int S0 = std::max(2, std::min(kMaxSplit, (sms - S * tiles) / (m->lay.n_out[0] / kBM)));
     plan.grad.n = L;
     plan.grad.z0[0] = 0;
     for (int l = 0; l < L; ++l) {
