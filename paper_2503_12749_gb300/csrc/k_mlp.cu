@@ -387,14 +387,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] = live ? silu_f(v[i]) : 0.0f;
             } else if (p.mode == kEpiLoss) {
-                float se = 0.0f;
+                // the row's 32 squared errors summed in a tree (a chain of 32 FP32
+                // additions errs by several times as much)
+                float sq[32];
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
                     const float e = live ? v[i] - tb[lane * kTurnRow + i] : 0.0f;
-                    se = fmaf(e, e, se);
+                    sq[i] = e * e;
                     v[i] = p.scale * e;
                 }
-                double s = (double)se;
+#pragma unroll
+                for (int w = 16; w > 0; w >>= 1)
+#pragma unroll
+                    for (int i = 0; i < w; ++i) sq[i] += sq[i + w];
+                double s = (double)sq[0];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                 if (lane == 0)

@@ -38,3 +38,19 @@ def test_weight_gradient_of_a_large_batch(gbs, width, batch):  # noqa: F811
     n = 3 * (batch // 8 // 16)
     loss = ((want - got) / want).median().item()
     assert abs(loss) <= n / 2 * 2.0**-23 + 1e-5, loss
+
+def test_loss_of_equal_errors(gbs):  # noqa: F811
+    """With zero weights and equal targets every squared error is the same FP32
+    number c.  Sums of 2, 4, .. 32 of them are exact in FP32, and so is the mean."""
+    import torch
+    dims = [10, 512, 512, 512]
+    params = [(np.zeros((dims[i + 1], dims[i])), np.zeros(dims[i + 1])) for i in range(3)]
+    mlp = gbs.gbs_mlp_create(10, 512, 512, 3, 1024)
+    gbs.gbs_mlp_set_params(mlp, np.concatenate([np.concatenate([W.ravel(), b]) for W, b in params]).astype(np.float32))
+    X = torch.randn(640, 10, device="cuda")
+    t = np.float32(1.2345678)
+    T = torch.full((640, 512), float(t), device="cuda")
+    loss, _ = gbs.gbs_mlp_gradients(mlp, X.data_ptr(), T.data_ptr(), 640)
+    gbs.gbs_mlp_free(mlp)
+    c = float(np.float32(t * t))
+    assert abs(loss - c) <= 2.0**-50 * c
