@@ -27,6 +27,7 @@ constexpr int kTrajBits = 3;
 // scales beyond 2^+-kExpRange are left to the SIMT kernel
 constexpr int kExpRange = 400;
 constexpr int kExpNone = -(1 << 20);
+constexpr int kExpVacuum = -kExpRange - 1;  // an input mode in the vacuum state
 
 // Byte offset of (row, k) within a slice of one 16-wide K step: 8-row groups
 // of 256 bytes, each two core matrices of 8 rows x 16 bytes.

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(256) k_f64tc_split_T(const double *__restrict_
     if (i < M)
         for (int j = threadIdx.x; j < N; j += 256) {
             const double v = src[j];
-            if (v != 0.0) ex = max(ex, ilogb(v) + 1 + col_exp[j]);
+            if (v != 0.0 && col_exp[j] != kExpVacuum) ex = max(ex, ilogb(v) + 1 + col_exp[j]);
         }
     ex = __reduce_max_sync(0xffffffffu, ex);
     if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = ex;
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(256) k_f64tc_split_T(const double *__restrict_
         int64_t x = 0;
         if (i < M && j < N) {
             const double v = src[j];
-            if (v != 0.0) x = to_fixed(v, 55 + col_exp[j] - ex);
+            if (v != 0.0 && col_exp[j] != kExpVacuum) x = to_fixed(v, 55 + col_exp[j] - ex);
         }
         uint32_t dg[kDigits];
         digit_pairs(x, 0, dg);
@@ -236,9 +236,9 @@ bool f64tc_column_exponents(const std::vector<double2> &sq, std::vector<int> &e)
     for (size_t j = 0; j < sq.size(); ++j) {
         const double h = 8.67 * std::hypot(sq[j].x, sq[j].y);
         if (!std::isfinite(h)) return false;
-        // an input in the vacuum state contributes nothing at any scale
-        e[j] = h > 0.0 ? std::ilogb(h) + 1 : -kExpRange;
-        if (e[j] < -kExpRange || e[j] > kExpRange) return false;
+        // an input in the vacuum state contributes nothing, whatever T couples to it
+        e[j] = h > 0.0 ? std::ilogb(h) + 1 : kExpVacuum;
+        if (h > 0.0 && (e[j] < -kExpRange || e[j] > kExpRange)) return false;
     }
     return true;
 }
