@@ -158,7 +158,8 @@ void net_free(gbs_net *net, T *&p) {
 bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
 int64_t pick_chunk(const gbs_net *net) {
-    // trajectories per chunk: sample operand <= 1 GiB, multiple of 128, in [128, 2^17]
+    // trajectories per chunk: sample operand <= 1 GiB (FP64 as digit tiles 1.75 GiB, 3.5
+    // where 16-mode padding doubles it), multiple of 128, in [128, 2^17]
     size_t per_traj;
     if (simt_precision(net->precision))
         per_traj = (size_t)16 * net->N;
@@ -578,6 +579,40 @@ int make_f64tc_operand(gbs_net *net, const std::vector<double2> &sq) {
     return GBS_OK;
 }
 
+// The chunk workspace from the stream-ordered pool; the sampler writes every
+// element the GEMM reads for valid trajectories (K padding included), so nothing
+// needs clearing.
+int alloc_workspace(gbs_net *net) {
+    if (simt_precision(net->precision)) {
+        net->B_bytes = net->d_Aq    ? f64tc_B_bytes(net->N, net->chunk)
+                       : net->d_T32 ? fp32_B_bytes(net->N, net->chunk)
+                                    : (size_t)net->chunk * 2 * net->N * sizeof(double);
+    } else {
+        const int64_t tiles = (net->chunk + kTcTileSamples - 1) / kTcTileSamples;
+        net->B_bytes = (size_t)net->planesB * tiles * 256 * net->ldK * sizeof(__nv_bfloat16);
+    }
+    int rc;
+    if ((rc = pool_alloc(&net->d_B, net->B_bytes, net->stream, "sample operand")) ||
+        (rc = pool_alloc_n(&net->d_n, (size_t)net->chunk, net->stream, "n")) ||
+        (rc = pool_alloc_n(&net->d_nS_part, (size_t)net->chunk * net->mtiles, net->stream, "nS_part")) ||
+        (rc = pool_alloc_n(&net->d_nS, (size_t)net->chunk, net->stream, "nS")) ||
+        (rc = pool_alloc_n(&net->d_win, (size_t)net->chunk, net->stream, "windows")) ||
+        (rc = net_alloc(net, &net->d_wmax, (size_t)2, "window union")) ||
+        (rc = net_alloc(net, &net->d_flags, (size_t)4, "flags")))
+        return rc;
+    return GBS_OK;
+}
+
+void free_workspace(gbs_net *net) {
+    pool_free(net->d_B, net->stream);
+    pool_free(net->d_n, net->stream);
+    pool_free(net->d_nS_part, net->stream);
+    pool_free(net->d_nS, net->stream);
+    pool_free(net->d_win, net->stream);
+    net_free(net, net->d_wmax);
+    net_free(net, net->d_flags);
+}
+
 // Shared by gbs_make_network (T in host memory) and gbs_make_network_device.
 int make_network(int N, int M, const double *T, bool T_device, const double *r, int precision,
                  void *stream, gbs_net_t *out) {
@@ -730,27 +765,25 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
             if (rc) return fail(rc);
         }
     }
-    // chunk workspace
     net->chunk = pick_chunk(net);
-    if (simt_precision(precision)) {
-        net->B_bytes = net->d_Aq    ? f64tc_B_bytes(N, net->chunk)
-                       : net->d_T32 ? fp32_B_bytes(N, net->chunk)
-                                 : (size_t)net->chunk * 2 * N * sizeof(double);
-    } else {
-        const int64_t tiles = (net->chunk + kTcTileSamples - 1) / kTcTileSamples;
-        net->B_bytes = (size_t)net->planesB * tiles * 256 * net->ldK * sizeof(__nv_bfloat16);
+    rc = alloc_workspace(net);
+    if (rc == GBS_ENOMEM && net->d_Aq) {
+        // the digit tiles take 1.75 times the doubles' room (and T's digits theirs):
+        // where that is missing the FMA kernel's operands, from T again
+        free_workspace(net);
+        net_free(net, net->d_Aq);
+        net_free(net, net->d_rowexp);
+        net_free(net, net->d_colexp);
+        if ((rc = net_alloc(net, &net->d_T64, (size_t)M * 2 * N, "T64")) ||
+            (rc = net_alloc(net, &d_bad, (size_t)1, "T check")))
+            return fail(rc);
+        k_t64_from_dev<<<conv_blocks, 256, 0, net->stream>>>(T, N, M, net->d_T64, d_bad);
+        net_free(net, d_bad);
+        rc = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(net->stream) == cudaSuccess
+                 ? alloc_workspace(net)
+                 : set_error(GBS_ECUDA, "conversion of T failed");
     }
-    // the chunk workspace from the stream-ordered pool; the sampler writes
-    // every element the GEMM reads for valid trajectories (K padding
-    // included), so nothing needs clearing
-    if ((rc = pool_alloc(&net->d_B, net->B_bytes, net->stream, "sample operand")) ||
-        (rc = pool_alloc_n(&net->d_n, (size_t)net->chunk, net->stream, "n")) ||
-        (rc = pool_alloc_n(&net->d_nS_part, (size_t)net->chunk * net->mtiles, net->stream, "nS_part")) ||
-        (rc = pool_alloc_n(&net->d_nS, (size_t)net->chunk, net->stream, "nS")) ||
-        (rc = pool_alloc_n(&net->d_win, (size_t)net->chunk, net->stream, "windows")) ||
-        (rc = net_alloc(net, &net->d_wmax, (size_t)2, "window union")) ||
-        (rc = net_alloc(net, &net->d_flags, (size_t)4, "flags")))
-        return fail(rc);
+    if (rc) return fail(rc);
     if (cudaMemsetAsync(net->d_flags, 0, 4 * sizeof(unsigned long long), net->stream) != cudaSuccess)
         return fail(set_error(GBS_ECUDA, "memset of flags failed"));
     if (!simt_precision(precision)) {
