@@ -203,14 +203,11 @@ void release_all(gbs_net *net) {
     release_estimator(net);
     prof_destroy(net);
     if (net->tc) tc_plan_destroy(net);
-    net_free(net, net->d_sq64);
-    net_free(net, net->d_sq32);
-    net_free(net, net->d_ntab);
+    net_free(net, net->d_setup);
     net_free(net, net->d_T64);
     net_free(net, net->d_T32);
     net_free(net, net->d_Aq);
     net_free(net, net->d_rowexp);
-    net_free(net, net->d_colexp);
     net_free(net, net->d_A);
     pool_free(net->d_B, net->stream);
     pool_free(net->d_B_alt, net->stream);
@@ -532,51 +529,35 @@ const char *gbs_last_error(void) { return error_message(); }
 namespace gbs {
 namespace {
 
-// Counts the non-finite entries found by one of the T conversion kernels.
-int finish_device_T(gbs_net *net, unsigned long long *d_bad) {
+// Reads what the T conversion kernels counted: non-finite entries, and (found,
+// may be NULL) rows outside the range of the FP64 digits.
+int finish_device_T(gbs_net *net, unsigned long long *d_bad, unsigned long long *rows = nullptr) {
     GBS_LAUNCH_CHECK();
-    unsigned long long bad = 0;
-    GBS_CUDA_TRY(cudaMemcpyAsync(&bad, d_bad, sizeof(bad), cudaMemcpyDeviceToHost, net->stream));
+    unsigned long long bad[2] = {0, 0};
+    GBS_CUDA_TRY(cudaMemcpyAsync(bad, d_bad, sizeof(bad), cudaMemcpyDeviceToHost, net->stream));
     GBS_CUDA_TRY(cudaStreamSynchronize(net->stream));
-    if (bad) return set_error(GBS_EINVAL, "T has %llu non-finite entries", bad);
+    if (bad[0]) return set_error(GBS_EINVAL, "T has %llu non-finite entries", bad[0]);
+    if (rows) *rows = bad[1];
     return GBS_OK;
 }
 
-// The operand of the FP64 GEMM on the tensor cores from d_T64, which is
-// released.  Networks whose squeezing or rows of T lie outside the range of
-// the digits' scales, or whose digits do not fit in memory, keep d_T64 and the
-// SIMT kernel.
-int make_f64tc_operand(gbs_net *net, const std::vector<double2> &sq) {
-    std::vector<int> e;
-    if (!f64tc_column_exponents(sq, e)) return GBS_OK;
+// Without the operand of the FP64 GEMM on the tensor cores the network runs the
+// FMA kernel.
+void drop_f64tc_operand(gbs_net *net) {
+    net_free(net, net->d_Aq);
+    net_free(net, net->d_rowexp);
+}
+
+// That operand from d_T64 (d_rows counts the rows of T outside the range of the
+// digits' scales); left out where it does not fit in memory.
+int start_f64tc_operand(gbs_net *net, unsigned long long *d_rows) {
     int rc;
-    unsigned long long *d_bad = nullptr, bad = 0;
-    auto drop = [&] {
-        net_free(net, net->d_Aq);
-        net_free(net, net->d_rowexp);
-        net_free(net, net->d_colexp);
-    };
-    if ((rc = net_alloc(net, &net->d_colexp, (size_t)net->N, "mode exponents")) ||
-        (rc = net_alloc(net, &net->d_rowexp, (size_t)net->mtiles * 128, "row exponents")) ||
-        (rc = net_alloc(net, &net->d_Aq, f64tc_A_bytes(net->N, net->mtiles), "digits of T")) ||
-        (rc = net_alloc(net, &d_bad, (size_t)1, "range check"))) {
-        drop();
+    if ((rc = net_alloc(net, &net->d_rowexp, (size_t)net->mtiles * 128, "row exponents")) ||
+        (rc = net_alloc(net, &net->d_Aq, f64tc_A_bytes(net->N, net->mtiles), "digits of T"))) {
+        drop_f64tc_operand(net);
         return rc == GBS_ENOMEM ? GBS_OK : rc;
     }
-    if (cudaMemcpyAsync(net->d_colexp, e.data(), sizeof(int) * net->N, cudaMemcpyHostToDevice,
-                        net->stream) != cudaSuccess ||
-        cudaMemsetAsync(d_bad, 0, sizeof(bad), net->stream) != cudaSuccess)
-        rc = set_error(GBS_ECUDA, "upload of the mode exponents failed");
-    if (!rc) rc = launch_f64tc_split_T(net, d_bad);
-    if (!rc && (cudaMemcpyAsync(&bad, d_bad, sizeof(bad), cudaMemcpyDeviceToHost, net->stream) !=
-                    cudaSuccess ||
-                cudaStreamSynchronize(net->stream) != cudaSuccess))
-        rc = set_error(GBS_ECUDA, "digits of T failed");
-    net_free(net, d_bad);
-    if (rc) return rc;
-    if (bad) drop();
-    else net_free(net, net->d_T64);
-    return GBS_OK;
+    return launch_f64tc_split_T(net, d_rows);
 }
 
 // The chunk workspace from the stream-ordered pool; the sampler writes every
@@ -674,6 +655,7 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
     net->stream = static_cast<cudaStream_t>(stream);
     int rc = GBS_OK;
     auto fail = [&](int code) {
+        cudaStreamSynchronize(net->stream);  // the upload's source goes out of scope
         release_all(net);
         delete net;
         return code;
@@ -697,20 +679,33 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
         sq64[j] = make_double2(std::sqrt(0.5 * sp), std::sqrt(0.5 * sm));
         sq32[j] = make_float2((float)sq64[j].x, (float)sq64[j].y);
     }
-    if ((rc = net_alloc(net, &net->d_sq64, (size_t)N, "sq64")) ||
-        (rc = net_alloc(net, &net->d_sq32, (size_t)N, "sq32")))
-        return fail(rc);
-    if (cudaMemcpyAsync(net->d_sq64, sq64.data(), sizeof(double2) * N, cudaMemcpyHostToDevice,
-                        net->stream) != cudaSuccess ||
-        cudaMemcpyAsync(net->d_sq32, sq32.data(), sizeof(float2) * N, cudaMemcpyHostToDevice,
-                        net->stream) != cudaSuccess ||
-        cudaStreamSynchronize(net->stream) != cudaSuccess)  // the host vectors go out of scope
+    // one upload: the coefficients, the tables of the FP64 normals (SIMT
+    // precisions), the input modes' exponents (FP64 as digits)
+    std::vector<int> col_exp;
+    const bool digits = precision == GBS_FP64 && N >= kF64tcMinN && f64tc_column_exponents(sq64, col_exp);
+    std::vector<uint8_t> setup;
+    auto put = [&](const void *src, size_t bytes) {
+        const size_t at = (setup.size() + 255) / 256 * 256;
+        setup.resize(at + bytes);
+        std::memcpy(setup.data() + at, src, bytes);
+        return at;
+    };
+    const size_t at64 = put(sq64.data(), sizeof(double2) * N), at32 = put(sq32.data(), sizeof(float2) * N);
+    const size_t at_tab = simt_precision(precision) ? put(norm_tab(), norm_tab_bytes()) : 0;
+    const size_t at_exp = digits ? put(col_exp.data(), sizeof(int) * N) : 0;
+    if ((rc = net_alloc(net, &net->d_setup, setup.size(), "sampler coefficients"))) return fail(rc);
+    net->d_sq64 = reinterpret_cast<double2 *>(net->d_setup + at64);
+    net->d_sq32 = reinterpret_cast<float2 *>(net->d_setup + at32);
+    net->d_ntab = at_tab ? reinterpret_cast<NormTab *>(net->d_setup + at_tab) : nullptr;
+    net->d_colexp = at_exp ? reinterpret_cast<int *>(net->d_setup + at_exp) : nullptr;
+    if (cudaMemcpyAsync(net->d_setup, setup.data(), setup.size(), cudaMemcpyHostToDevice, net->stream) !=
+        cudaSuccess)
         return fail(set_error(GBS_ECUDA, "upload of sampler coefficients failed"));
 
     unsigned long long *d_bad = nullptr;
     if (T_device) {
-        if ((rc = net_alloc(net, &d_bad, (size_t)1, "T check"))) return fail(rc);
-        if (cudaMemsetAsync(d_bad, 0, sizeof(unsigned long long), net->stream) != cudaSuccess) {
+        if ((rc = net_alloc(net, &d_bad, (size_t)2, "T check"))) return fail(rc);
+        if (cudaMemsetAsync(d_bad, 0, 2 * sizeof(unsigned long long), net->stream) != cudaSuccess) {
             net_free(net, d_bad);
             return fail(set_error(GBS_ECUDA, "memset failed"));
         }
@@ -723,21 +718,20 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
             return fail(rc);
         }
         k_t64_from_dev<<<conv_blocks, 256, 0, net->stream>>>(T, N, M, net->d_T64, d_bad);
-        rc = finish_device_T(net, d_bad);
+        // (the digits are formed before T has been found finite: one synchronisation)
+        rc = digits ? start_f64tc_operand(net, d_bad + 1) : GBS_OK;
+        unsigned long long rows = 0;
+        if (!rc) rc = finish_device_T(net, d_bad, &rows);
         net_free(net, d_bad);
         if (rc) return fail(rc);
-        if ((rc = pool_alloc(reinterpret_cast<void **>(&net->d_ntab), norm_tab_bytes(), net->stream,
-                             "normal tables")) ||
-            (rc = upload_norm_tab(net)))
-            return fail(rc);
+        if (rows) drop_f64tc_operand(net);
+        if (net->d_Aq) net_free(net, net->d_T64);
         if (precision == GBS_FP32) {
             if ((rc = net_alloc(net, &net->d_T32, fp32_A_floats(N, net->mtiles), "T32")) ||
                 (rc = launch_t32_tiles(net)))
                 return fail(rc);
             net_free(net, net->d_T64);
         }
-        if (precision == GBS_FP64 && N >= kF64tcMinN && (rc = make_f64tc_operand(net, sq64)))
-            return fail(rc);
     } else {
         // A = [Re T_i.; Im T_i.] rows interleaved per output mode, T rounded to
         // FP32 and split into BF16 planes T = T0 + T1 + T2, each plane
@@ -771,9 +765,7 @@ int make_network(int N, int M, const double *T, bool T_device, const double *r, 
         // the digit tiles take 1.75 times the doubles' room (and T's digits theirs):
         // where that is missing the FMA kernel's operands, from T again
         free_workspace(net);
-        net_free(net, net->d_Aq);
-        net_free(net, net->d_rowexp);
-        net_free(net, net->d_colexp);
+        drop_f64tc_operand(net);
         if ((rc = net_alloc(net, &net->d_T64, (size_t)M * 2 * N, "T64")) ||
             (rc = net_alloc(net, &d_bad, (size_t)1, "T check")))
             return fail(rc);

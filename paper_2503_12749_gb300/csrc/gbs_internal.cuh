@@ -156,6 +156,8 @@ struct gbs_net {
     cudaStream_t stream = nullptr;
     int device = 0, sm_count = 0;
 
+    // one buffer of what set-up uploads: d_sq64, d_sq32, d_ntab, d_colexp
+    uint8_t *d_setup = nullptr;
     // per-mode sampler coefficients: (sqrt(s+/2), sqrt(s-/2)), s+- = sinh r e^{+-r}
     double2 *d_sq64 = nullptr;
     float2 *d_sq32 = nullptr;
@@ -270,8 +272,8 @@ void pool_free_raw(void *p, cudaStream_t stream);
 // Sampler: writes the sample operand for trajectories e0..e0+count-1 and n[].
 int launch_sample_fp64(gbs_net *net, uint64_t seed, uint64_t e0, int64_t count);
 int launch_sample_bf16(gbs_net *net, uint64_t seed, uint64_t e0, int64_t count);
-// The FP64 normals' tables into net->d_ntab.
-int upload_norm_tab(gbs_net *net);
+// The FP64 normals' tables (host; net->d_ntab holds a copy).
+const NormTab *norm_tab();
 size_t norm_tab_bytes();
 // The BF16 sampler's job for trajectories e0..e0+count-1 into (B, n).
 SampleJob sample_job_bf16(gbs_net *net, void *B, double *n, uint64_t seed, uint64_t e0,

@@ -270,14 +270,13 @@ int launch_sample_fp64(gbs_net *net, uint64_t seed, uint64_t e0, int64_t count) 
     return GBS_OK;
 }
 
-int upload_norm_tab(gbs_net *net) {
+const NormTab *norm_tab() {
     static const NormTab T = [] {
         NormTab t;
         fill_norm_tab(t);
         return t;
     }();
-    GBS_CUDA_TRY(cudaMemcpyAsync(net->d_ntab, &T, sizeof(T), cudaMemcpyHostToDevice, net->stream));
-    return GBS_OK;
+    return &T;
 }
 
 size_t norm_tab_bytes() { return sizeof(NormTab); }
