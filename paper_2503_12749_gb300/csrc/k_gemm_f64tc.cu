@@ -183,48 +183,84 @@ __global__ void __launch_bounds__(kThreads, 1)
     pipe.close(tmem);
 }
 
-// One block per row (mode i, Re or Im) of the padded operand: the row's
-// scale, then its digits.  bad counts the rows whose scale lies outside the
-// range the digits are used for.
-__global__ void __launch_bounds__(256) k_f64tc_split_T(const double *__restrict__ T64,
-                                                       const int *__restrict__ col_exp, int N,
-                                                       int M, int KB, uint8_t *__restrict__ A,
-                                                       int *__restrict__ row_exp,
-                                                       unsigned long long *__restrict__ bad) {
-    __shared__ int s_max[8];
-    const int row = blockIdx.x;
-    const int i = row >> 1;
-    const double *src = T64 + ((size_t)i * 2 + (row & 1)) * N;
-    int ex = kExpNone;
-    if (i < M)
-        for (int j = threadIdx.x; j < N; j += 256) {
-            const double v = src[j];
-            if (v != 0.0 && col_exp[j] != kExpVacuum) ex = max(ex, ilogb(v) + 1 + col_exp[j]);
-        }
-    ex = __reduce_max_sync(0xffffffffu, ex);
-    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = ex;
-    __syncthreads();
-    ex = s_max[0];
+// One block per 8 rows (a row of core matrices) and 256 k of the padded operand: the
+// rows' scales, a warp each, then the digits of 8 consecutive k of a row per thread,
+// so that a digit's 8 rows are one 128-byte store.  bad counts the rows whose scale
+// lies outside the range the digits are used for.  Bound by latency, so every load of
+// a thread is in flight at once and the scales are formed again in each of a row's
+// blocks: N = M = 1000 24 us; a row per block with 16-bit stores 43, loads one by one
+// and FP64 comparisons 36.
+constexpr int kSplitRows = 8;
+// (integer instructions: an FP64 comparison takes 16 clocks of a warp)
+__device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
+__device__ __forceinline__ int exponent_of(double v) {  // ilogb for v != 0
+    const int e = (__double2hiint(v) >> 20) & 0x7ff;
+    return e ? e - 1023 : ilogb(v);
+}
+__global__ void __launch_bounds__(32 * kSplitRows)
+    k_f64tc_split_T(const double *__restrict__ T64, const int *__restrict__ col_exp, int N, int M,
+                    int KB, uint8_t *__restrict__ A, int *__restrict__ row_exp,
+                    unsigned long long *__restrict__ bad) {
+    __shared__ int s_ex[kSplitRows];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int row0 = blockIdx.x * kSplitRows;
+    {
+        const int row = row0 + warp, i = row >> 1;
+        const double *src = T64 + ((size_t)i * 2 + (row & 1)) * N;
+        int ex = kExpNone;
+        for (int j0 = lane; i < M && j0 < N; j0 += 256) {
+            double v[8];
+            int e[8];
 #pragma unroll
-    for (int w = 1; w < 8; ++w) ex = max(ex, s_max[w]);
-    if (ex == kExpNone) ex = 0;
-    if (threadIdx.x == 0) {
-        row_exp[row] = ex;
-        if (ex < -kExpRange || ex > kExpRange) atomicAdd(bad, 1ull);
+            for (int t = 0; t < 8; ++t) {
+                const int j = j0 + 32 * t;
+                v[t] = j < N ? src[j] : 0.0;
+                e[t] = j < N ? col_exp[j] : kExpVacuum;
+            }
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                if (nonzero(v[t]) && e[t] != kExpVacuum) ex = max(ex, exponent_of(v[t]) + 1 + e[t]);
+        }
+        ex = __reduce_max_sync(0xffffffffu, ex);
+        if (ex == kExpNone) ex = 0;
+        if (lane == 0) s_ex[warp] = ex;
+        if (lane == 0 && blockIdx.y == 0) {
+            row_exp[row] = ex;
+            if (ex < -kExpRange || ex > kExpRange) atomicAdd(bad, 1ull);
+        }
     }
+    __syncthreads();
+    const int row = row0 + (threadIdx.x & (kSplitRows - 1)), i = row >> 1;
+    const int ex = s_ex[threadIdx.x & (kSplitRows - 1)];
+    const double *src = T64 + ((size_t)i * 2 + (row & 1)) * N;
     uint8_t *tile = A + (size_t)(row >> 7) * KB * kAStage;
-    const int r = row & 127;
-    for (int j = threadIdx.x; j < KB * 16; j += 256) {
-        int64_t x = 0;
-        if (i < M && j < N) {
-            const double v = src[j];
-            if (v != 0.0 && col_exp[j] != kExpVacuum) x = to_fixed(v, 55 + col_exp[j] - ex);
-        }
-        uint32_t dg[kDigits];
-        digit_pairs(x, 0, dg);
-        uint8_t *p = tile + (size_t)(j >> 4) * kAStage + core_offset(r, j & 15);
+    const int g = blockIdx.y * 32 + threadIdx.x / kSplitRows;  // group of 8 k
+    if (g < 2 * KB) {
+        double v[8];
+        int e[8];
 #pragma unroll
-        for (int q = 0; q < kDigits; ++q) *reinterpret_cast<uint16_t *>(p + q * kASlice) = (uint16_t)dg[q];
+        for (int t = 0; t < 8; ++t) {  // every load in flight at once
+            const int j = 8 * g + t;
+            const bool in = i < M && j < N;
+            v[t] = in ? src[j] : 0.0;
+            e[t] = in ? col_exp[j] : kExpVacuum;
+        }
+        uint32_t dg[kDigits][4];
+#pragma unroll
+        for (int t = 0; t < 8; t += 2) {
+            int64_t x[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                x[h] = nonzero(v[t + h]) && e[t + h] != kExpVacuum ? to_fixed(v[t + h], 55 + e[t + h] - ex) : 0;
+            uint32_t d[kDigits];
+            digit_pairs(x[0], x[1], d);
+#pragma unroll
+            for (int q = 0; q < kDigits; ++q) dg[q][t >> 1] = d[q];
+        }
+        uint8_t *p = tile + (size_t)(g >> 1) * kAStage + core_offset(row & 127, 8 * (g & 1));
+#pragma unroll
+        for (int q = 0; q < kDigits; ++q)
+            *reinterpret_cast<uint4 *>(p + q * kASlice) = make_uint4(dg[q][0], dg[q][1], dg[q][2], dg[q][3]);
     }
 }
 
@@ -252,7 +288,8 @@ size_t f64tc_B_bytes(int N, int64_t chunk) {
 int launch_f64tc_split_T(gbs_net *net, unsigned long long *d_bad) {
     GBS_CUDA_TRY(cudaFuncSetAttribute(k_gemm_f64tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       kSmemBytes));
-    k_f64tc_split_T<<<net->mtiles * 128, 256, 0, net->stream>>>(
+    const dim3 grid((unsigned)(net->mtiles * 128 / kSplitRows), (unsigned)((2 * f64tc_kblocks(net->N) + 31) / 32));
+    k_f64tc_split_T<<<grid, 32 * kSplitRows, 0, net->stream>>>(
         net->d_T64, net->d_colexp, net->N, net->M, f64tc_kblocks(net->N), net->d_Aq, net->d_rowexp,
         d_bad);
     GBS_LAUNCH_CHECK();
