@@ -72,8 +72,8 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
 // block's own mean, which k_sur_features joins (Chan, Golub, LeVeque, "Algorithms
 // for computing the sample variance", Amer. Statist. 37, 1983): nothing cancels,
 // whatever c is.
-// part[net][chunk] = sum r - c, sum (r - c - its chunk mean)^2, sum sinh^2,
-// sum sinh^4, min, max.
+// part[net][chunk] = sum r - c, sum (r - c - its chunk mean)^2, sum eta sinh^2, sum
+// (eta sinh^2)^2 (finite wherever the variance is), min, max.
 constexpr int kFeatChunk = 512;
 constexpr int kFeatPart = 6;
 
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256) k_sur_feature_parts(const NetIn *__restri
     const int j0 = blockIdx.x * kFeatChunk;
     if (j0 >= n.N) return;
     const double *rj = r + n.r0;
-    const double c = rj[0];
+    const double c = rj[0], eta = n.t * n.t;
     double v[kFeatPart] = {0.0, 0.0, 0.0, 0.0, INFINITY, -INFINITY};
     auto join = [](double (&a)[kFeatPart], const double (&b)[kFeatPart]) {
 #pragma unroll
@@ -101,9 +101,9 @@ __global__ void __launch_bounds__(256) k_sur_feature_parts(const NetIn *__restri
         const double x = rj[j];
         const double u = expm1(x);
         const double sh = 0.5 * (u + (u < 0x1p60 ? u / (u + 1.0) : 1.0));
-        const double sh2 = sh * sh;
+        const double m = eta * (sh * sh);
         dev[t] = x - c;
-        join(v, {dev[t], 0.0, sh2, sh2 * sh2, x, x});
+        join(v, {dev[t], 0.0, m, m * m, x, x});
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -157,9 +157,9 @@ __global__ void k_sur_features(const NetIn *__restrict__ nets, const double *__r
 #pragma unroll
     for (int q = 0; q < kFeatPart; ++q) t[q] = __shfl_sync(0xffffffffu, v, q);
     const double eta = n.t * n.t;
-    const double mu = eta * t[2];
+    const double mu = t[2];
     // sum of eta sinh^2 + eta^2 sinh^2 (1 + 2 sinh^2)
-    const double s = sqrt(mu + eta * mu + 2.0 * eta * eta * t[3]);
+    const double s = sqrt(mu + eta * mu + 2.0 * t[3]);
     const double d = t[0] / (double)n.N;
     // the chunk means' own deviations, a chunk per lane
     double between = 0.0;
