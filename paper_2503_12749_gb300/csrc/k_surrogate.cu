@@ -384,12 +384,15 @@ int gbs_surrogate_features(int count, const int *N, const int *M, const double *
     int Nmax = 0;
     for (int i = 0; i < count; ++i) Nmax = N[i] > Nmax ? N[i] : Nmax;
     const int chunks = (Nmax + kFeatChunk - 1) / kFeatChunk;
-    // Where the device addresses pageable host memory (Grace), r is read in
-    // place, once, over the host link; else it is uploaded.  The call
-    // synchronises before it returns, so r is not read afterwards.
+    // Where the device reads the host's own page tables (Grace), r is read in place,
+    // once, over the host link; else it is uploaded: also where pageable memory is
+    // addressable but its pages would migrate, and an r that is not 8-byte aligned.
+    // The call synchronises before it returns, so r is not read afterwards.
     int dev = 0, direct = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&direct, cudaDevAttrPageableMemoryAccess, dev) != cudaSuccess) {
+    if (reinterpret_cast<uintptr_t>(r) % sizeof(double) == 0 &&
+        (cudaGetDevice(&dev) != cudaSuccess ||
+         cudaDeviceGetAttribute(&direct, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev) !=
+             cudaSuccess)) {
         cudaGetLastError();
         direct = 0;
     }
