@@ -874,11 +874,6 @@ __global__ void __launch_bounds__(kGfSlots * kGfGroups, GBS_GF_MINBLOCKS)
 
 }  // namespace
 
-namespace {
-
-
-}  // namespace
-
 Gf64Tables make_gf64_tables() {
     Gf64Tables T;
     // long double exceeds double on both host architectures; elsewhere the
@@ -981,14 +976,20 @@ int launch_gf(gbs_net *net, uint64_t e0, int64_t count) {
     if (count <= 0) return GBS_OK;
     if (simt_precision(net->precision)) {
         static const Gf64Tables T = make_gf64_tables();
-        // Blocks per sub-ensemble: enough for 8 blocks per SM with up to 11
-        // blocks of pair slots (what the windows of a 1000-mode network
-        // leave), each half-warp keeping at least 16 trajectories
+        // Blocks per sub-ensemble: four per SM, each half-warp keeping at least 16
+        // trajectories.  Blocks of pair slots that the windows leave: the terms
+        // beyond 1 - cos theta = 60 ln 2 / n_S are skipped, and a circle holds about four
+        // times the mean count, so theta K1 / 2 pi = 2.9 sqrt(K1) pairs.  Measured (us, C =
+        // 1, 2, 4, 8; the rule's in brackets), modes / sub-ensembles / K1: 16 / 16 / 64 432
+        // 227 209 [166]; 1000 / 100 / 4096 [604] 608 709 895; 615 x 700 / 37 / 2048 827 [688]
+        // 727 776; 400 / 20 / 4096 1325 1337 [1360] 1374; 1500 / 10 / 8192 358 279 [248] 246;
+        // 60 / 30 / 1024 659 573 [561] 633; 100 / 10 / 512 3626 3212 2851 [2814].
         const int slots = (net->K1 / 2 + 1 + kG64Slots - 1) / kG64Slots;
+        const int left = std::min(slots, 1 + (int)(2.9 * std::sqrt((double)net->K1) / kG64Slots));
         const int64_t per = count / net->n_sub / kG64Groups;
         int C = 1;
         while (C < kG64MaxCluster && per >= 32 * C &&
-               (int64_t)net->n_sub * C * std::min(slots, 11) < 8 * (int64_t)net->sm_count)
+               (int64_t)net->n_sub * C * left < 4 * (int64_t)net->sm_count)
             C *= 2;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(net->n_sub * C), (unsigned)slots);
