@@ -88,9 +88,10 @@ GF_FP32_OPS_PER_PAIR = 200.5
 # 1.057 TFLOP/s on GB300, below the 1.25 a plain FP64 GEMM (k_gemm_fp64)
 # sustains on m8000 (8MN FLOP per trajectory over CUDA-event kernel time), so
 # the larger of the probe and GB300's nominal FP64 rate is the FP64 pipe's peak.
-# The FP64 path's GEMM (k_gemm_f64tc) forms its products as 34 exact digit
-# products on the tensor cores and exceeds it.
+# From 16 input modes the FP64 path's GEMM (k_gemm_f64tc) forms its products as 34
+# exact digit products on the tensor cores, whose bound is their 16-bit rate / 34.
 F64TC_PRODUCTS = 34
+F64TC_MIN_MODES = 16
 FP64_NOMINAL_TFLOPS = 1.25
 # FP32 FMA peak from unit counts: 152 SMs x 128 FP32 lanes x 2 FLOP x 2.07 GHz
 FP32_UNIT_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
@@ -442,12 +443,14 @@ def gbs_arm(args, wl_def):
     else:
         achieved = flops / (gemm_ms / 1e3) / 1e12
         probe = gbs.gbs_measure_fp64_rate(sptr)
-        peak = max(probe, FP64_NOMINAL_TFLOPS)
-        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak if peak else None, "traffic": None,
-                "kernel": "k_gemm_f64tc", "fp64_probe_tflops": probe,
-                "digit_products_tflops": achieved * F64TC_PRODUCTS,
-                "peak_source": FP64_PEAK_SOURCE}
+        digits = netdef.N >= F64TC_MIN_MODES  # else FP64 FMAs (k_gemm_fp64)
+        peak = peaks["bf16_tflops"] / F64TC_PRODUCTS if digits else max(probe, FP64_NOMINAL_TFLOPS)
+        roof = {"bound": "tensor" if digits else "alu", "achieved": achieved, "peak": peak,
+                "unit": "TFLOP/s", "frac": achieved / peak if peak else None, "traffic": None,
+                "kernel": "k_gemm_f64tc" if digits else "k_gemm_fp64", "fp64_probe_tflops": probe,
+                "digit_products_tflops": achieved * F64TC_PRODUCTS if digits else None,
+                "peak_source": (f"{peak_kind} 16-bit rate (burst) / {F64TC_PRODUCTS} digit products"
+                                if digits else FP64_PEAK_SOURCE)}
     phases = {k: {"ms_per_step": v[0] / args.steps, "launches_per_step": v[1] / args.steps}
               for k, v in prof.items()}
     launches = int(sum(v[1] for v in prof.values()))
@@ -532,8 +535,8 @@ def gbs_arm(args, wl_def):
             "gemm_ms": fp64_gemm_ms, "gemm_tflops": fp64_gemm_tflops,
             "fp64_peak_tflops": fp64_peak, "fp64_probe_tflops": fp64_probe,
             "fp64_peak_source": FP64_PEAK_SOURCE,
-            "gemm_frac_of_fp64_peak": fp64_gemm_tflops / fp64_peak if fp64_peak else None,
             "gemm_digit_products_tflops": fp64_gemm_tflops * F64TC_PRODUCTS,
+            "gemm_frac_of_digit_product_peak": fp64_gemm_tflops * F64TC_PRODUCTS / peaks["bf16_tflops"],
             "speedup_of_split_path": value / (Ef / (ms64 / 1e3)),
             "max_abs_dP_over_sigma_fp64": float(np.max(np.abs(Pb[0] - P64[0]) / sig)),
             "max_abs_dP_plusP_over_sigma_fp64": float(np.max(np.abs(Pb[2] - P64[2]) /

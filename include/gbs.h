@@ -53,8 +53,10 @@ extern "C" {
 #define GBS_ENOTSUP (-6)    /* feature not supported on this device / build */
 
 /* Arithmetic of the propagation GEMM alpha' = T alpha, beta' = T* beta. */
-#define GBS_FP64 0   /* FP64 sampler, FP64 SIMT GEMM, FP64 generating functions */
-#define GBS_FP32 1   /* as GBS_FP64 with the SIMT GEMM in FP32: T and the samples
+#define GBS_FP64 0   /* FP64 sampler, FP64 GEMM (exact products of 56- and 58-bit
+                        fixed-point operands on the tensor cores from 16 input
+                        modes, FP64 FMAs otherwise), FP64 generating functions */
+#define GBS_FP32 1   /* as GBS_FP64 with a SIMT GEMM in FP32: T and the samples
                         rounded to FP32, FP32 products accumulated in FP32 along
                         the N input modes; occupations and everything after
                         them in FP64 */

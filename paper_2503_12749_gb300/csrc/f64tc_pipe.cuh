@@ -256,11 +256,10 @@ struct Pipe {
         __syncwarp();
         ptx::tc_fence_after();
         // 8 columns at a time: the sums hold 128 registers.  The other sub-tile's
-        // turn (kBurst stages, 2176 clocks) covers this; the conversions' 16 lanes
-        // per clock take 2048 for eight sums, so D_0 and D_1, which are below
-        // 2^22, get theirs from an addition of 1.5 2^23, and D_0 2^8 + D_1 and
-        // D_2 2^8 + D_3 (below 2^31: d + 1 digit pairs of 2^21 each) share a
-        // 64-bit addition.
+        // turns (kBurst stages each, 2176 clocks) run meanwhile, but do not cover this
+        // entirely: the conversions' 16 lanes per clock take 2048 for eight sums, so
+        // D_0 and D_1, which are below 2^22, get theirs from an addition of 1.5 2^23,
+        // and D_0 2^8 + D_1 and D_2 2^8 + D_3 (below 2^31) share a 64-bit addition.
 #pragma unroll
         for (int c0 = 0; c0 < 32; c0 += 8) {
             float u[8], v[8];

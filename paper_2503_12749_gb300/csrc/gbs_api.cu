@@ -1369,7 +1369,7 @@ int gbs_set_gemm_config(gbs_net_t net, int pair, int band, int keep_a) {
     int rc;
     if ((rc = validate_net(net))) return rc;
     if (simt_precision(net->precision))
-        return set_error(GBS_EINVAL, "the FP64 and FP32 paths have no tcgen05 GEMM");
+        return set_error(GBS_EINVAL, "the tile configuration is the BF16 GEMM's");
     GemmCfg c;
     c.pair = pair;
     c.band = band;

@@ -105,7 +105,7 @@ __device__ __forceinline__ double transpose_sum(double (&v)[16], int lane) {
 
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_f64tc(const uint8_t *__restrict__ A, const uint8_t *__restrict__ B,
-                 const int *__restrict__ row_exp, int KB, int M, int mtiles, int stiles,
+                 const int *__restrict__ row_exp, int KB, int mtiles, int stiles,
                  int64_t count, int64_t ld_part, double2 *__restrict__ nS_part, OccOut64 occ,
                  uint64_t wait_ns, unsigned long long *err_ptr) {
     extern __shared__ uint8_t smem_raw[];
@@ -304,7 +304,7 @@ int launch_gemm_f64tc(gbs_net *net, int64_t count, OccOut64 occ) {
     const int grid = (int)std::min<int64_t>(ntiles, net->sm_count);
     k_gemm_f64tc<<<grid, kThreads, kSmemBytes, net->stream>>>(
         net->d_Aq, static_cast<const uint8_t *>(net->d_B), net->d_rowexp, f64tc_kblocks(net->N),
-        net->M, net->mtiles, (int)stiles, count, net->chunk, net->d_nS_part, occ, net->wait_ns,
+        net->mtiles, (int)stiles, count, net->chunk, net->d_nS_part, occ, net->wait_ns,
         net->d_flags + 1);
     GBS_LAUNCH_CHECK();
     return GBS_OK;

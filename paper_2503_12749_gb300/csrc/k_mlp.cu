@@ -643,7 +643,6 @@ struct gbs_mlp {
     float *lr = nullptr;
     int lr_cap = 0;
     float *loss_hist = nullptr;
-    int hist_cap = 0;
     double *loss64 = nullptr;
     unsigned long long *err = nullptr;
 };
@@ -1107,7 +1106,6 @@ int gbs_mlp_train(gbs_mlp_t m, const float *X_dev, const float *T_dev, int batch
         float *h = nullptr;
         if ((rc = mlp_alloc(&h, (size_t)steps, m->owned))) return rc;
         m->loss_hist = h;
-        m->hist_cap = steps;
     }
     GBS_CUDA_TRY(cudaMemcpyAsync(m->lr, lr, sizeof(float) * steps, cudaMemcpyHostToDevice, m->stream));
     GBS_CUDA_TRY(cudaMemsetAsync(m->step + 1, 0, sizeof(long long), m->stream));
