@@ -14,7 +14,7 @@
 // conversion from FP64 is done once, not once per tile.  Measured at 700 x 615,
 // 20001 trajectories: 3.75 ms for the FP64 kernel's tiling with FP32 registers
 // (64 x 32 tile, 4 x 2 modes by trajectories per thread, operands converted as
-// they were staged) -> 1.45 ms (50 TFLOP/s over the padded tiles, 0.61 of the pipe).
+// they were staged) -> 1.09 ms (66 TFLOP/s over the padded tiles, 0.82 of the pipe).
 #include "gbs_internal.cuh"
 #include "tc_ptx.cuh"
 

@@ -199,8 +199,8 @@ __device__ __forceinline__ void pair_slot_to_k(int i, int K1, int W1, int W2, bo
 // cluster: one thread per k walking all of them left a 64-point circle to 1024
 // threads.  Measured (ms, before -> now): N = 16, K1 = 64, 16384 trajectories in 16
 // sub-ensembles 2.39 -> 0.16; N = 1000, K1 = 4096, 32768 in 100 3.60 -> 0.61
-// (5.3e6 pairs, 0.56 of the FP64 pipe); a 615 x 700 network with complex n_S,
-// K1 = 2048, 20001 in 37 2.63 -> 0.74.
+// (FP64 pipe 84 % busy); a 615 x 700 network with complex n_S,
+// K1 = 2048, 20001 in 37 2.63 -> 0.69.
 // ---------------------------------------------------------------------------
 constexpr int kG64Slots = 16;   // mirror pairs per block, the lanes of each half-warp
 constexpr int kG64Groups = 8;   // half-warps per block, splitting the trajectories

@@ -20,6 +20,11 @@
 // (e^kSepTcTop64), or whose phase or exponent is beyond the double-float functions,
 // are listed for the general kernels (k_gf2d_df, k_gf2d).  The integer sums do not depend on
 // their order, so the lists are compacted.
+// Root mean square error over the grid of the mean sums of 160 trajectories against
+// 113-bit arithmetic from the same n and n_Sb (matrix-P, +P; general kernels -> here):
+// FP64, 8 modes 1.2e-16, 4.8e-16 -> 5.0e-17, 3.3e-16; 40 4.6e-17, 3.6e-17 -> 3.7e-17,
+// 2.2e-17; 200 lossless (9 networks) 1.6e-16, 2.2e-17 -> 1.5e-16, 1.5e-17; BF16, 8
+// modes 1.6e-14, 1.0e-14 -> 2.8e-15, 5.5e-15; 200 lossy 3.0e-16, 3.0e-16 -> 1.5e-16, 1.5e-16.
 //
 // Why: the double-float outer products are 2 x 16 packed FP32 instructions per
 // grid point and trajectory on the FP32 pipe; as digits they are 34 tensor-core
